@@ -23,7 +23,8 @@
 // reduces them in a fixed order and computes the next pass's coefficients,
 // alpha, beta and the breakdown flag on the device - no host round trip.
 //
-// Precision: DDD uses binary64 FMA.  FDF stores V in binary32 and carries
+// Precision: DDD uses binary64 FMA (and binary32 for updates whose terms all
+// lie below 2^-36 of the result, see low_coefs).  FDF stores V in binary32 and carries
 // every product and sum in double-float (te_common.cuh); per-CTA partials are
 // double-float, the final cross-CTA sums binary64.
 #include "te_common.cuh"
@@ -95,13 +96,20 @@ constexpr int GROUP_MIN_PER_CTA = 8;
 
 __host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// DDD updates: a column's small coefficients in binary32 (scaled), and the
+// exponent that brings its elements into binary32's range
+struct __align__(16) LowCoef {
+  float c1, c2;
+  int bias, pad_;
+};
+
 struct SmemPlan {
-  size_t region, ws_off, coef_off, coef2_off, ritz_off, red_off, fin_off, bar_off, total;
+  size_t region, ws_off, coef_off, coef2_off, ritz_off, red_off, fin_off, low_off, bar_off, total;
 };
 // finalize scratch (doubles): copies of s, alpha, beta, the c_j, warp sums
 constexpr int FIN_SCRATCH = 4 * (MAX_M + 2) + 2 * (CONSUMERS / 32) + 8;
 // ritz_elems: m*K coefficients held by the Ritz pass (0 for the other passes)
-__host__ __device__ inline SmemPlan smem_plan(int mode, size_t region, int ritz_elems) {
+__host__ __device__ inline SmemPlan smem_plan(int prec, int mode, size_t region, int ritz_elems) {
   SmemPlan p{};
   p.region = region;
   p.ws_off = align_up(region, 128);
@@ -111,8 +119,10 @@ __host__ __device__ inline SmemPlan smem_plan(int mode, size_t region, int ritz_
   size_t ritz = (mode == MODE_RITZ) ? align_up((size_t)ritz_elems * 8, 128) : 0;
   p.red_off = p.ritz_off + ritz;
   p.fin_off = align_up(p.red_off + PSTRIDE * 8, 8);
-  p.bar_off = p.fin_off + FIN_SCRATCH * 8;
-  p.total = p.bar_off + 2 * MAX_STAGES * 8 + 16;
+  p.low_off = align_up(p.fin_off + FIN_SCRATCH * 8, alignof(LowCoef));
+  p.bar_off = align_up(
+      p.low_off + (prec == PREC_DDD && mode != MODE_RITZ ? sizeof(LowCoef) * MAX_M : 0), 8);
+  p.total = p.bar_off + 2 * MAX_STAGES * 8 + 32;
   return p;
 }
 
@@ -184,6 +194,108 @@ template <int P>
 TE_DEV double acc_to_double(typename PassTr<P>::acc_t a) {
   if constexpr (P == PREC_FDF) return dw_to_double(dacc_value(a));
   else return a;
+}
+
+// ---------------------------------------------------------------------------
+// DDD updates: small coefficients in binary32
+// ---------------------------------------------------------------------------
+// An update subtracts c_j times column j.  Once the sweeps have made the basis
+// orthogonal, all but the last two coefficients sit at the rounding level (of
+// the order of 1e-15), and their products need only a few digits: where every
+// one of them is below 2^LOW_BITS of the update's scale, the products are
+// taken in binary32 (error 2^-24 2^LOW_BITS = 2^-60 of that scale, under the
+// binary64 rounding of the exact terms), off the binary64 pipe that would
+// bind the pass; otherwise in binary64 as before.  The scale: the largest
+// term of the update itself (the alpha and beta terms), |alpha| + beta for
+// the second sweep of a stored vector, the candidate for its own correction.
+// Elements are scaled by their column's bound, so that binary32 holds them
+// whatever the matrix's magnitude; exponents outside what that covers, zero
+// scales and NaN take the binary64 form.  One warp per CTA, integers only.
+// R-MAT 2^22, 16 columns on average: the delayed form's update 284 -> 125 us
+// (5.25 TB/s; the binary64 pipe was 83 % busy at 27 % of the DRAM peak), the
+// solve 40.5 -> 34.9 ms; the Lanczos phase of 2^19 rows and 40 steps with both
+// sweeps 9.58 -> 8.52 ms.  Error against 64 bits unchanged (4.3e-14 and 5.0e-14
+// for the former's vectors, 1.2e-15 for the latter's basis).
+constexpr int LOW_BITS = -36;
+
+TE_DEV int biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// a bound on the (biased) exponents of a column with scale s = 1 / norm
+TE_DEV int column_exp(double s) { return 2046 - biased_exp(s); }
+// binary64 to binary32 with its exponent lowered by `bias` (>> 20), truncated;
+// what falls below the range becomes about 2^-126
+TE_DEV float low_word(double x, int bias) {
+  const int hi = __double2hiint(x);
+  const int a = max((hi & 0x7fffffff) - bias, 0);
+  const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)a, 3);
+  return __uint_as_float((b & 0x7fffffffu) | ((unsigned)hi & 0x80000000u));
+}
+
+// f times 2^r as binary64, exact for normal f (|r| <= LOW_EXP)
+constexpr int LOW_EXP = 800;
+TE_DEV double low_result(float f, int r) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  const unsigned hi = (b & 0x80000000u) | ((m >> 3) + ((unsigned)(896 + r) << 20));
+  return m < 0x00800000u ? 0.0 : __hiloint2double((int)hi, (int)(m << 29));
+}
+
+template <int MODE>
+TE_DEV void low_coefs(const PassArgs& a, LowCoef* lc, int* info, int lane) {
+  const LzState* st = a.st;
+  constexpr bool DUPD = MODE == MODE_DCGS_UPDATE;
+  const int ncol = DUPD ? a.nb - 1 : a.nb;             // columns with coefficients
+  const int nexact = DUPD ? 1 : a.exact_tail;          // the last ones stay in binary64 (c2)
+  const int nsmall = ncol > nexact ? ncol - nexact : 0;
+  const double* c1 = DUPD ? st->c1 : nullptr;
+  const double* c2 = MODE == MODE_AXPY_DOT ? st->c1 : st->c2;
+  // biased exponent of |c| times the column's bound; 0 for c = 0
+  int ref = 0, ref1 = 0, worst = 0, worst1 = 0, emin = 2046, emax = 0;
+  if (DUPD) {
+    const int ec = column_exp(st->s[a.col0 + a.nb - 1]);
+    ref1 = 1023 + ec;
+    ref = st->f2 != 0.0 ? biased_exp(st->f2) + ec : 0;
+    emin = emax = ec;
+  }
+  if (MODE == MODE_AXPY_STORE)
+    ref = biased_exp(fabs(st->alpha[a.step]) + st->beta[a.step]) + 1023;
+  bool fine = true;
+  for (int j = lane; j < ncol; j += 32) {
+    const int ec = column_exp(st->s[a.col0 + j]);
+    const int b2 = biased_exp(c2[j]), k2 = b2 > 0 ? b2 + ec : 0;
+    const int b1 = DUPD ? biased_exp(c1[j]) : 0, k1 = b1 > 0 ? b1 + ec : 0;
+    fine &= b1 < 0x7ff && b2 < 0x7ff;
+    ref = max(ref, k2);
+    if (j < nsmall) worst = max(worst, k2);
+    worst1 = max(worst1, k1);
+    emin = min(emin, ec);
+    emax = max(emax, ec);
+  }
+  ref = __reduce_max_sync(0xffffffffu, ref);
+  worst = __reduce_max_sync(0xffffffffu, worst);
+  worst1 = __reduce_max_sync(0xffffffffu, worst1);
+  emin = __reduce_min_sync(0xffffffffu, emin);
+  emax = __reduce_max_sync(0xffffffffu, emax);
+  // results are scaled by 2^r (update) and 2^r1 (the candidate's correction)
+  const int r = ref - 2046, r1 = ref1 - 2046;
+  fine = __all_sync(0xffffffffu, fine) && nsmall > 0 && emin >= 128 && emax <= 2000 && ref > 0 &&
+         worst <= ref + LOW_BITS && r >= -LOW_EXP && r <= LOW_EXP;
+  if (DUPD)
+    fine = fine && worst1 <= ref1 + LOW_BITS && r1 >= -LOW_EXP && r1 <= LOW_EXP;
+  if (lane == 0) {
+    info[0] = fine;
+    info[1] = r;
+    info[2] = r1;
+  }
+  if (!fine) return;  // uniform
+  for (int j = lane; j < ncol; j += 32) {
+    const int ec = column_exp(st->s[a.col0 + j]);
+    LowCoef o;
+    // c 2^(ec - 1023 - r): at most 2^LOW_BITS where it is used
+    o.c2 = j < nsmall && c2[j] != 0.0 ? low_word(c2[j], (896 + r - (ec - 1023)) * (1 << 20)) : 0.f;
+    o.c1 = DUPD && c1[j] != 0.0 ? low_word(c1[j], (896 + r1 - (ec - 1023)) * (1 << 20)) : 0.f;
+    o.bias = (ec - 127) * (1 << 20);  // an element times 2^-(ec - 1023), below 1 in magnitude
+    o.pad_ = 0;
+    lc[j] = o;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -404,7 +516,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
     if (*((volatile int*)&st->restart_flag) == 0) return;
   }
   const SmemPlan L = smem_plan(
-      MODE, region, MODE == MODE_RITZ ? a.nb * ((a.K + RITZ_KC - 1) / RITZ_KC * RITZ_KC) : 0);
+      P, MODE, region, MODE == MODE_RITZ ? a.nb * ((a.K + RITZ_KC - 1) / RITZ_KC * RITZ_KC) : 0);
   vec_t* ws = reinterpret_cast<vec_t*>(sm + L.ws_off);
   coef_t* coef = reinterpret_cast<coef_t*>(sm + L.coef_off);
   coef_t* coef2 = reinterpret_cast<coef_t*>(sm + L.coef2_off);
@@ -472,6 +584,11 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
       coef[j] = to_coef<P>(st->c1[j]);
       coef2[j] = to_coef<P>(st->c2[j]);
     }
+  }
+  LowCoef* lowc = reinterpret_cast<LowCoef*>(sm + L.low_off);
+  int* lowinfo = abortflag + 1;  // whether the small coefficients go in binary32; two exponents
+  if constexpr (P == PREC_DDD && (HAS_AXPY || DUPD)) {
+    if (wid == 0) low_coefs<MODE>(a, lowc, lowinfo, lane);
   }
   // Ritz coefficients C (nb x K) with the row stride padded to Kp (a multiple
   // of RITZ_KC, zeros beyond K); FDF keeps their binary32 roundings only
@@ -554,6 +671,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
   for (int q = 0; q < QMAX; ++q) dots[q] = zero_acc<P>();
 #pragma unroll
   for (int q = 0; q < (DDOT ? QMAX : 1); ++q) dots2[q] = zero_acc<P>();
+  const bool low = P == PREC_DDD && (HAS_AXPY || DUPD) && lowinfo[0] != 0;
   acc_t n1 = zero_acc<P>(), n2 = zero_acc<P>();
   basis_t* Vout = static_cast<basis_t*>(a.Vmut) + (size_t)a.col_out * a.cstride;
 
@@ -621,6 +739,23 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
           for (; j < nsmall; ++j) f[0] = __fmaf_rn(tv[(size_t)j * TILE_R + tid], coef[j].x, f[0]);
           tacc = dacc_zero();
           dacc_add_pair(tacc, __fadd_rn(f[0], f[1]), __fadd_rn(f[2], f[3]));
+          for (; j < nb; ++j) acc_fma<P>(tacc, tv[(size_t)j * TILE_R + tid], coef[j]);
+        } else if (low) {
+          const int nsmall = nb - a.exact_tail;  // > 0
+          float f[4] = {0.f, 0.f, 0.f, 0.f};
+          int j = 0;
+          for (; j + 4 <= nsmall; j += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const LowCoef lc = lowc[j + u];
+              f[u] = __fmaf_rn(low_word(tv[(size_t)(j + u) * TILE_R + tid], lc.bias), lc.c2, f[u]);
+            }
+          }
+          for (; j < nsmall; ++j) {
+            const LowCoef lc = lowc[j];
+            f[0] = __fmaf_rn(low_word(tv[(size_t)j * TILE_R + tid], lc.bias), lc.c2, f[0]);
+          }
+          tacc = low_result(__fadd_rn(__fadd_rn(f[0], f[1]), __fadd_rn(f[2], f[3])), lowinfo[1]);
           for (; j < nb; ++j) acc_fma<P>(tacc, tv[(size_t)j * TILE_R + tid], coef[j]);
         } else {
           acc_t ta[4] = {zero_acc<P>(), zero_acc<P>(), zero_acc<P>(), zero_acc<P>()};
@@ -724,10 +859,33 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
           dacc_fma(n2, w.x, w.x, 0.0f);
         } else {
           double t1 = 0.0, t2 = 0.0;
-          for (int j = 0; j < nj; ++j) {
-            const double v = tv[(size_t)j * TILE_R + tid];
-            t1 = fma(v, coef[j], t1);
-            t2 = fma(v, coef2[j], t2);
+          if (low) {  // (nj >= 2: the beta term is column nj - 1)
+            float f[2] = {0.f, 0.f}, g[2] = {0.f, 0.f};
+            int j = 0;
+            for (; j + 2 <= nj; j += 2) {
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const LowCoef lc = lowc[j + u];
+                const float v = low_word(tv[(size_t)(j + u) * TILE_R + tid], lc.bias);
+                f[u] = __fmaf_rn(v, lc.c1, f[u]);
+                g[u] = __fmaf_rn(v, lc.c2, g[u]);
+              }
+            }
+            if (j < nj) {
+              const LowCoef lc = lowc[j];
+              const float v = low_word(tv[(size_t)j * TILE_R + tid], lc.bias);
+              f[0] = __fmaf_rn(v, lc.c1, f[0]);
+              g[0] = __fmaf_rn(v, lc.c2, g[0]);
+            }
+            t1 = low_result(__fadd_rn(f[0], f[1]), lowinfo[2]);
+            t2 = low_result(__fadd_rn(g[0], g[1]), lowinfo[1]);
+            t2 = fma(tv[(size_t)(nj - 1) * TILE_R + tid], coef2[nj - 1], t2);
+          } else {
+            for (int j = 0; j < nj; ++j) {
+              const double v = tv[(size_t)j * TILE_R + tid];
+              t1 = fma(v, coef[j], t1);
+              t2 = fma(v, coef2[j], t2);
+            }
           }
           t2 = fma(sc, fcand, t2);
           if (nj > 0) Vfix[vrow] = sc - t1;
@@ -1157,7 +1315,7 @@ static cudaError_t config_t(int max_cols, int K, int num_sms, PassLaunch& out) {
   const int ritz_elems = MODE == MODE_RITZ ? max_cols * ((K + RITZ_KC - 1) / RITZ_KC * RITZ_KC) : 0;
   // pass_ctas_per_sm CTAs per SM share the SM's shared memory (minus the
   // per-CTA reservation of 1 KB)
-  const size_t fixed = smem_plan(MODE, 0, ritz_elems).total + 128;
+  const size_t fixed = smem_plan(P, MODE, 0, ritz_elems).total + 128;
   int persm = 0;
   e = cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e != cudaSuccess) return e;
@@ -1172,7 +1330,7 @@ static cudaError_t config_t(int max_cols, int K, int num_sms, PassLaunch& out) {
   const size_t region = avail / 128 * 128;
   const int stages = (int)(region / per_stage);
   if (stages < 1) return cudaErrorInvalidConfiguration;
-  const size_t total = smem_plan(MODE, region, ritz_elems).total;
+  const size_t total = smem_plan(P, MODE, region, ritz_elems).total;
   e = cudaFuncSetAttribute(pass_kernel<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)total);
   if (e != cudaSuccess) return e;
