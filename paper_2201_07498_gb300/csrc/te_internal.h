@@ -331,23 +331,19 @@ cudaError_t jacobi_prepare();  // once per process/device, outside stream captur
 cudaError_t launch_jacobi(const JacobiArgs& a, cudaStream_t s);
 
 // ---- Rayleigh-quotient refinement and Gram matrix ----
-// For Ritz vector k (st->eigvecs + k*n) and y = M u_k (binary64): replaces
-// st->theta_sel[k] by the Rayleigh quotient theta + u'r/u'u (r = y - theta u)
-// and st->resid_est[k] by ||y - theta' u|| / ||u||; also writes
-// st->eigvals_out[k] when set.  `partials`: grid * 4 doubles.
-cudaError_t launch_refine(LzState* st, const double* y, int64_t n, int k, double* partials,
-                          int grid, cudaStream_t s);
+// The K Ritz vectors U (binary64, by rows, row stride K rounded up to even)
+// against the binary64 matrix S: replaces st->theta_sel[k] by the Rayleigh
+// quotient theta + u'r/u'u (r = M u - theta u) and st->resid_est[k] by ||M u -
+// theta' u|| / ||u||; also writes st->eigvals_out[k] when set.  `pieces`: the
+// layout's cut-row pieces; `scratch`: at least 2 KB, 16-byte aligned; `filled`:
+// n bytes; *kernels: the kernels launched.
+cudaError_t launch_refine(LzState* st, const DevSell& S, int64_t n, int K, const double* U,
+                          int64_t pieces, void* scratch, size_t scratch_bytes,
+                          unsigned char* filled, int num_sms, int* kernels, cudaStream_t s);
 int refine_grid(int num_sms);
-// copy `count` doubles from src to st->eigvecs_user (no-op when it is NULL)
-cudaError_t launch_copy_out(LzState* st, const double* src, size_t count, int grid,
-                            cudaStream_t s);
-// st->eigvecs_user[k*n + v] = src[k*n + iperm[v]] for k < K, v < n: Ritz
-// vectors of the relabelled rows back in the caller's row order (no-op when
-// eigvecs_user is NULL)
-cudaError_t launch_copy_out_perm(LzState* st, const double* src, int64_t n, int K,
-                                 const int32_t* iperm, int grid, cudaStream_t s);
-// the same from vectors stored by rows: st->eigvecs_user[k*n + v] =
-// src[iperm[v] * Kr + k], Kr = K rounded up to even
+// the Ritz vectors, stored by rows, into the caller's columns and row order:
+// st->eigvecs_user[k*n + v] = src[iperm[v] * Kr + k], Kr = K rounded up to even
+// (iperm NULL: v); no-op when eigvecs_user is NULL
 cudaError_t launch_copy_out_rows(LzState* st, const double* src, int64_t n, int K,
                                  const int32_t* iperm, int grid, cudaStream_t s);
 // G[a*K + b] = u_a . u_b (device), per-block partials in `partials`

@@ -114,12 +114,19 @@ Work layout(int prec, int vk, int64_t n_pad, int m, int grid, const SellSizes& z
   w.V = take((size_t)n_pad * (size_t)(m + 1) * basis_elt(prec));
   w.ytil = take((size_t)n_pad * 8);
   w.xcur = take((size_t)n_pad * basis_elt(prec));
-  w.w = take((size_t)n_pad * 8);
   w.partials = take((size_t)grid * PSTRIDE * 8);
   w.st = take(sizeof(LzState));
-  // by rows (K rounded up to even) for relabelled rows without refinement
-  const size_t kcols = (reorder && !refine) ? (size_t)((K + 1) & ~1) : (size_t)K;
-  w.Uint = (refine || reorder) ? take((size_t)n * kcols * 8) : 0;
+  w.w = take((size_t)n_pad * 8);
+  // by rows, K rounded up to even; with refinement and an odd K the vectors
+  // start where w lies (n_pad binary64, which the Ritz pass no longer needs and
+  // every solve writes before it reads), so the last column costs no memory
+  const size_t even = (size_t)((K + 1) & ~1);
+  if (refine && (K & 1)) {
+    w.Uint = w.w;
+    off = std::max(off, al256(w.w + (size_t)n * even * 8));
+  } else {
+    w.Uint = (refine || reorder) ? take((size_t)n * even * 8) : 0;
+  }
   w.perm = reorder ? take((size_t)n * 4) : 0;
   w.iperm = reorder ? take((size_t)n * 4) : 0;
   w.slices = take(std::max<size_t>(z.slices, 1) * sizeof(SellSlice));
@@ -209,7 +216,8 @@ struct te_plan {
   cudaStream_t cs = nullptr;   // copy stream
   cudaEvent_t ev_ready[2] = {nullptr, nullptr}, ev_free[2] = {nullptr, nullptr};
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  double* ubase = nullptr;  // with refinement or reordering: the plan's Ritz vectors (n x K)
+  double* ubase = nullptr;  // with refinement or reordering: the plan's Ritz vectors, by rows
+  int64_t npieces = 0;      // pieces of cut rows in the SpMV layout
   bool reorder = false;     // rows relabelled by degree (te_options.order)
   int32_t* dperm = nullptr;   // solver row r = caller row dperm[r] (device)
   int32_t* diperm = nullptr;  // its inverse
@@ -663,7 +671,7 @@ cudaError_t enqueue_solve(te_plan* P, cudaStream_t s) {
   PassArgs a = base_args(P);
   a.nb = P->m;
   a.fin = FIN_NONE;
-  if (P->reorder && !P->refine) a.urows = P->ubase;  // stored by rows, gathered below
+  if (P->reorder || P->refine) a.urows = P->ubase;  // stored by rows, gathered below
   if ((e = pass(P, MODE_RITZ, a, s)) != cudaSuccess) return e;
   const int rgrid = refine_grid(P->num_sms);
   if (!P->refine) {
@@ -676,25 +684,24 @@ cudaError_t enqueue_solve(te_plan* P, cudaStream_t s) {
       return e;
     return prof_end(P, s, TE_KIND_RITZ, (16.0 + 4.0 / P->K) * (double)P->n * P->K);
   }
-  // binary64 Rayleigh-quotient refinement: y = M u_k, then the reduction
-  double* y = static_cast<double*>(at(P, P->W.ytil));
-  double* part = static_cast<double*>(at(P, P->W.partials));
-  for (int k = 0; k < P->K; ++k) {
-    P->nkernels += 2 + (P->sell64.nlrows > 0 ? 1 : 0);
-    if ((e = prof_begin(P, s)) != cudaSuccess) return e;
-    e = launch_spmv(PREC_DDD, P->sell64, P->ubase + (size_t)k * P->n, y, true, s);
-    if (e != cudaSuccess) return e;
-    if ((e = launch_refine(P->st, y, P->n, k, part, rgrid, s)) != cudaSuccess) return e;
-    const double n = (double)P->n, nnz = (double)P->nnz;
-    if ((e = prof_end(P, s, TE_KIND_REFINE, nnz * 12.0 + 8.0 * (n + 1.0) + 8.0 * n * 3.0)) !=
-        cudaSuccess)
-      return e;
-  }
+  // binary64 Rayleigh-quotient refinement.  Its scratch: the basis (the Ritz
+  // pass was its last reader, and every solve writes a column before it reads
+  // it), and the contiguous column for the rows' marks.
+  if ((e = prof_begin(P, s)) != cudaSuccess) return e;
+  int kern = 0;
+  e = launch_refine(P->st, P->sell64, P->n, P->K, P->ubase, P->npieces, at(P, P->W.V),
+                    (size_t)P->n_pad * (size_t)(P->m + 1) * basis_elt(P->prec),
+                    static_cast<unsigned char*>(at(P, P->W.xcur)), P->num_sms, &kern, s);
+  if (e != cudaSuccess) return e;
+  P->nkernels += kern;
+  const double dn = (double)P->n, dnnz = (double)P->nnz;
+  if ((e = prof_end(P, s, TE_KIND_REFINE,
+                    dnnz * 12.0 + 8.0 * (dn + 1.0) + 8.0 * dn * P->K)) != cudaSuccess)
+    return e;
   // the refined vectors stay the Ritz vectors: hand them to the caller's buffer
   P->nkernels++;
   if ((e = prof_begin(P, s)) != cudaSuccess) return e;
-  e = P->reorder ? launch_copy_out_perm(P->st, P->ubase, P->n, P->K, P->diperm, rgrid * 4, s)
-                 : launch_copy_out(P->st, P->ubase, (size_t)P->n * P->K, rgrid * 4, s);
+  e = launch_copy_out_rows(P->st, P->ubase, P->n, P->K, P->diperm, rgrid * 4, s);
   if (e != cudaSuccess) return e;
   return prof_end(P, s, TE_KIND_REFINE, 16.0 * (double)P->n * P->K);
 }
@@ -1187,6 +1194,7 @@ te_status te_plan_create(const te_csr* A, int32_t K, int32_t krylov_steps, te_pr
   P->sell.nslices = (int)l_slices;
   P->sell.nlrows = (int)l_lrows;
   P->sell.nlbig = (int)sell.nbig;  // (the device build sets it below)
+  P->npieces = l_pieces;
   void* vals64 = P->W.svals64 ? at(P, P->W.svals64) : nullptr;
   P->sell.vk = P->vk;
   P->sell.hot = P->reorder ? P->n : 0;  // the first columns are the most connected
