@@ -81,6 +81,44 @@ TE_DEV double dw_to_double_bits(dw v) {
   return __longlong_as_double((long long)(((uint64_t)(hb >> 31) << 63) | mag));
 }
 
+// Conversions by integer operations, for finite values.  x >= 0 to binary32,
+// truncated (0 below 2^-126); and what that leaves, truncated to 23 bits
+// (x in [2^-102, 2^128), else 0).
+TE_DEV float f_head(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const unsigned b = __funnelshift_l((unsigned)lo, (unsigned)(hi - (896 << 20)), 3);
+  return hi < (897 << 20) ? 0.f : __uint_as_float(b);
+}
+TE_DEV float f_tail(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned rem = ((unsigned)__double2loint(x) & 0x1fffffffu) >> 6;
+  const unsigned e = ((unsigned)(hi >> 20) - 896u - 23u) << 23;
+  return hi < (921 << 20) ? 0.f : __uint_as_float(e | rem) - __uint_as_float(e);
+}
+// binary32 to binary64, exact (subnormals become zero)
+TE_DEV double f_wide(float f) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  const unsigned hi = (b & 0x80000000u) | ((m >> 3) + (896u << 20));
+  return m < 0x00800000u ? 0.0 : __hiloint2double((int)hi, (int)(m << 29));
+}
+// x to binary32, truncated towards zero, either sign
+TE_DEV float f_narrow(double x) {
+  const unsigned sign = (unsigned)__double2hiint(x) & 0x80000000u;
+  return __uint_as_float(__float_as_uint(f_head(fabs(x))) | sign);
+}
+
+// binary64 to binary32, round to nearest even (the integer form for results in
+// binary32's normal range, where a carry out of the largest is infinity)
+TE_DEV float f32_from_f64(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u > 1150u - 897u) return __double2float_rn(x);
+  const unsigned b = __funnelshift_l(lo, (hi & 0x7fffffffu) - (896u << 20), 3);
+  const unsigned rem = lo & 0x1fffffffu, half = 0x10000000u;
+  const unsigned up = (rem > half || (rem == half && (b & 1u))) ? 1u : 0u;
+  return __uint_as_float((b + up) | (hi & 0x80000000u));
+}
+
 // AccurateDWPlusDW (Joldes et al. 2017, Alg. 6): relative error <= 3u^2
 TE_DEV dw dw_add(dw x, dw y) {
   float sh, sl, th, tl;

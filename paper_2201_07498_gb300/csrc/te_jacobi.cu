@@ -124,32 +124,6 @@ TE_DEV bool sel_before(int64_t a, int ia, int64_t b, int ib, int which) {
 // |x| as an integer that orders like it
 TE_DEV int64_t abs_bits(double x) { return __double_as_longlong(x) & INT64_MAX; }
 
-// Conversions by integer operations, for finite values.  x >= 0 to binary32,
-// truncated (0 below 2^-126); and what that leaves, truncated to 23 bits
-// (x in [2^-102, 2^128), else 0).
-TE_DEV float f_head(double x) {
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const unsigned b = __funnelshift_l((unsigned)lo, (unsigned)(hi - (896 << 20)), 3);
-  return hi < (897 << 20) ? 0.f : __uint_as_float(b);
-}
-TE_DEV float f_tail(double x) {
-  const int hi = __double2hiint(x);
-  const unsigned rem = ((unsigned)__double2loint(x) & 0x1fffffffu) >> 6;
-  const unsigned e = ((unsigned)(hi >> 20) - 896u - 23u) << 23;
-  return hi < (921 << 20) ? 0.f : __uint_as_float(e | rem) - __uint_as_float(e);
-}
-// binary32 to binary64, exact (subnormals become zero)
-TE_DEV double f_wide(float f) {
-  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
-  const unsigned hi = (b & 0x80000000u) | ((m >> 3) + (896u << 20));
-  return m < 0x00800000u ? 0.0 : __hiloint2double((int)hi, (int)(m << 29));
-}
-// x to binary32, truncated towards zero, either sign
-TE_DEV float f_narrow(double x) {
-  const unsigned sign = (unsigned)__double2hiint(x) & 0x80000000u;
-  return __uint_as_float(__float_as_uint(f_head(fabs(x))) | sign);
-}
-
 // The rotation that annihilates t_pq: t = tan of the angle, c = 1 / sqrt(1 +
 // t^2), s = t c.  With A = |t_pq| and D = |t_qq - t_pp|, |t| is the root of
 // A t^2 + D t - A in (0, 1], and 2 A t + D = sqrt(D^2 + 4 A^2) there, the

@@ -27,10 +27,10 @@
 
 namespace te {
 
-// Vin -> Vout: binary64 -> binary32 rounds to nearest even (__double2float_rn)
+// Vin -> Vout: binary64 -> binary32 rounds to nearest even
 template <typename Vin, typename Vout>
 TE_DEV Vout convert_value(Vin v) {
-  if constexpr (sizeof(Vin) == 8 && sizeof(Vout) == 4) return __double2float_rn(v);
+  if constexpr (sizeof(Vin) == 8 && sizeof(Vout) == 4) return f32_from_f64(v);
   else return (Vout)v;
 }
 
