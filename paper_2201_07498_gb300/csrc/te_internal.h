@@ -166,7 +166,7 @@ struct DevLayout {
   const int64_t* view_src = nullptr;
   const int32_t* view_len = nullptr;
   const int32_t* view_perm = nullptr;
-  int64_t nslices = 0, entries = 0, pieces = 0, nlrows = 0;
+  int64_t nslices = 0, entries = 0, pieces = 0, nlrows = 0, longest = 0;
   // err receives the reason when the row pointers are malformed or the size
   // is not covered (cudaErrorInvalidValue is returned then)
   cudaError_t count(const int64_t* rp_dev, int64_t n, int64_t nnz, int window, int vmax,

@@ -15,13 +15,19 @@
 // digits among the lanes with __match_any_sync so that equal keys keep their
 // input order.
 //
-// Arrangement: a warp per window of rows.  Counting: the histogram of piece
-// lengths gives the window's slices, padded entries, cut-row pieces and cut
-// rows; an exclusive scan over the windows places them.  Emission: the
-// window's rows are walked in order, 32 at a time; full-length pieces take
-// consecutive positions of their length class (warp prefix sums), shorter
-// pieces are ranked within their class with __match_any_sync, so every piece
-// lands at the position a stable sort by length (longest first) gives it.
+// Arrangement: a CTA per window of rows, its warps taking consecutive shares of
+// the rows.  Counting: each warp counts its pieces by length; the window's
+// totals give its slices, padded entries, cut-row pieces and cut rows; an
+// exclusive scan over the windows places them.  Emission: the warps' counts,
+// scanned over the warps, give each warp its first position in every length
+// class; it walks its rows in order, 32 at a time: full-length pieces take
+// consecutive positions of their class (warp prefix sums), shorter pieces are
+// ranked within their class with __match_any_sync, so every piece lands at
+// the position a stable sort by length (longest first) gives it.  Bound: the
+// latency of the walk (a warp per window walked 64 groups of rows, and all
+// pieces of the hub rows of a power-law matrix, one after another: counting and
+// emission 236 + 844 us for 1 M rows with cliques, under 20 + 61 us now; 128 +
+// 168 us for five windows of 10,007 rows, under 20 each now).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -38,7 +44,9 @@ namespace {
 constexpr int DS_TILE = 2048;  // elements per warp and pass
 constexpr int DS_WARPS = 8;    // warps per CTA
 constexpr int DS_BINS = 256;
-constexpr int LD_WARPS = 8;    // warps (windows) per CTA of the arrangement kernels
+constexpr int LD_WARPS = 16;   // most warps of a window's CTA (a window's rows / 64, at least one)
+constexpr int LD_BIG = 64;     // rows of a window whose pieces the whole CTA writes
+constexpr int LD_BIG_PIECES = 256;  // ... those with more full pieces than this
 constexpr int LD_MAX_VMAX = 128;
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 4;  // elements per thread of a scan block
@@ -94,11 +102,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_sums_kernel(const int64_t* 
   }
 }
 
-// exclusive scan of `cnt` values in one block (cnt <= SCAN_BLOCK); the total
-// goes to *total
+// exclusive scan of `cnt` values per block (cnt <= SCAN_BLOCK): block b takes
+// the b-th `cnt` values, and their total goes to total[b]
 __global__ void __launch_bounds__(SCAN_THREADS) scan_one_block_kernel(int64_t* a, int64_t cnt,
                                                                       int64_t* total) {
   __shared__ int64_t ws[SCAN_THREADS / 32];
+  a += blockIdx.x * cnt;
+  if (total) total += blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   int64_t v[SCAN_ITEMS];
   int64_t mine = 0;
@@ -296,48 +306,122 @@ TE_DEV void row_pieces(int64_t L, int vmax, int64_t& nfull, int& s) {
   }
 }
 
-// WinCount fields as four int64 arrays (slices, entries, pieces, lrows),
-// one entry per window
-__global__ void __launch_bounds__(32 * LD_WARPS) win_count_kernel(RowsView R, int64_t n,
-                                                                  int window, int vmax,
-                                                                  int64_t nwin, int64_t* wc) {
-  __shared__ int64_t hist[LD_WARPS][LD_MAX_VMAX + 1];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t win = (int64_t)blockIdx.x * LD_WARPS + w;
-  if (win >= nwin) return;  // uniform per warp
-  for (int l = lane; l <= vmax; l += 32) hist[w][l] = 0;
+int ld_warps(int window) { return std::min(std::max(window / 64, 1), LD_WARPS); }
+
+// What a window's CTA shares.  Lengths run from 1 to vmax; class vmax holds the
+// full pieces of every row, class l < vmax the last pieces of length l.
+struct WinShared {
+  unsigned cnt[LD_WARPS][LD_MAX_VMAX + 1];  // a warp's pieces by length (l < vmax)
+  int64_t full[LD_WARPS];                   // its full pieces
+  int64_t cutp[LD_WARPS];                   // its pieces of cut rows
+  int64_t cut[LD_WARPS];                    // its cut rows
+  int64_t start[LD_MAX_VMAX + 2];           // first sorted position of a length
+  int64_t ebase[LD_MAX_VMAX + 2];           // entries of the slices of longer lengths
+  int64_t np, entries;                      // the window's pieces and padded entries
+};
+
+// Counts (a warp per share of the rows) and the classes' positions.  Every
+// thread; ends with a barrier.
+TE_DEV void win_classes(const RowsView& R, int64_t r0, int64_t r1, int64_t s0, int64_t s1,
+                        int vmax, WinShared& S) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int l = lane; l <= vmax; l += 32) S.cnt[w][l] = 0;
   __syncwarp();
-  const int64_t r0 = win * window, r1 = r0 + window < n ? r0 + window : n;
-  int64_t pieces = 0, lrows = 0, np = 0;
-  for (int64_t r = r0 + lane; r < r1; r += 32) {
-    const int64_t L = R.L(r);
+  int64_t full = 0, cutp = 0, cut = 0;
+  for (int64_t c0 = s0; c0 < s1; c0 += 32) {
+    const int64_t r = c0 + lane;
+    const int64_t L = r < s1 ? R.L(r) : 0;
     int64_t nfull;
     int s;
     row_pieces(L, vmax, nfull, s);
-    if (nfull) atomicAdd(reinterpret_cast<unsigned long long*>(&hist[w][vmax]),
-                         (unsigned long long)nfull);
-    if (s) atomicAdd(reinterpret_cast<unsigned long long*>(&hist[w][s]), 1ull);
-    np += nfull + (s ? 1 : 0);
+    full += nfull;
     if (L > vmax) {
-      pieces += nfull + (s ? 1 : 0);
-      lrows += 1;
+      cutp += nfull + (s ? 1 : 0);
+      cut += 1;
+    }
+    const unsigned peers = __match_any_sync(0xffffffffu, s);
+    if (s && lane == __ffs(peers) - 1) S.cnt[w][s] += __popc(peers);
+    __syncwarp();
+  }
+  full = warp_isum(full);
+  cutp = warp_isum(cutp);
+  cut = warp_isum(cut);
+  if (lane == 0) {
+    S.full[w] = full;
+    S.cutp[w] = cutp;
+    S.cut[w] = cut;
+  }
+  __syncthreads();
+  if (w == 0) {
+    constexpr int PER = (LD_MAX_VMAX + 31) / 32;  // lengths per lane, longest first
+    int64_t c[PER];
+    int64_t mine = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int l = vmax - (lane * PER + i);
+      c[i] = 0;
+      if (l >= 1)
+        for (int q = 0; q < nw; ++q) c[i] += l == vmax ? S.full[q] : (int64_t)S.cnt[q][l];
+      mine += c[i];
+    }
+    int64_t np;
+    int64_t at = warp_excl_scan(mine, &np);
+    int64_t first[PER], ent[PER], esum = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int l = vmax - (lane * PER + i);
+      first[i] = at;
+      const int64_t n0 = (at + SELL_C - 1) / SELL_C;
+      at += c[i];
+      ent[i] = l >= 1 ? ((at + SELL_C - 1) / SELL_C - n0) * SELL_C * l : 0;
+      esum += ent[i];
+    }
+    int64_t etot;
+    int64_t eat = warp_excl_scan(esum, &etot);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int l = vmax - (lane * PER + i);
+      if (l >= 1) {
+        S.start[l] = first[i];
+        S.ebase[l] = eat;
+      }
+      eat += ent[i];
+    }
+    if (lane == 0) {
+      S.np = np;
+      S.entries = etot;
     }
   }
-  pieces = warp_isum(pieces);
-  lrows = warp_isum(lrows);
-  np = warp_isum(np);
-  __syncwarp();
-  if (lane == 0) {
-    int64_t at = 0, entries = 0;
-    for (int L = vmax; L >= 1; --L) {
-      const int64_t h = hist[w][L];
-      if (h == 0) continue;
-      const int64_t starts = (at + h + SELL_C - 1) / SELL_C - (at + SELL_C - 1) / SELL_C;
-      entries += starts * SELL_C * L;
-      at += h;
+  __syncthreads();
+}
+
+// a warp's share of the window's rows (a multiple of 32 but for the last)
+TE_DEV void win_share(int64_t r0, int64_t r1, int64_t& s0, int64_t& s1) {
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int64_t per = ((r1 - r0 + nw - 1) / nw + 31) / 32 * 32;
+  s0 = r0 + w * per < r1 ? r0 + w * per : r1;
+  s1 = s0 + per < r1 ? s0 + per : r1;
+}
+
+// window counts as four int64 arrays (slices, entries, pieces, lrows), one
+// entry per window
+__global__ void __launch_bounds__(32 * LD_WARPS) win_count_kernel(RowsView R, int64_t n,
+                                                                  int window, int vmax,
+                                                                  int64_t nwin, int64_t* wc) {
+  __shared__ WinShared S;
+  const int64_t win = blockIdx.x;
+  const int64_t r0 = win * window, r1 = r0 + window < n ? r0 + window : n;
+  int64_t s0, s1;
+  win_share(r0, r1, s0, s1);
+  win_classes(R, r0, r1, s0, s1, vmax, S);
+  if (threadIdx.x == 0) {
+    int64_t pieces = 0, lrows = 0;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
+      pieces += S.cutp[q];
+      lrows += S.cut[q];
     }
-    wc[win] = (np + SELL_C - 1) / SELL_C;
-    wc[nwin + win] = entries;
+    wc[win] = (S.np + SELL_C - 1) / SELL_C;
+    wc[nwin + win] = S.entries;
     wc[2 * nwin + win] = pieces;
     wc[3 * nwin + win] = lrows;
   }
@@ -348,69 +432,63 @@ __global__ void __launch_bounds__(32 * LD_WARPS) win_emit_kernel(
     RowsView R, int64_t n, int window, int vmax, int64_t nwin, const int64_t* off,
     SellSlice* slices, int32_t* vout, int64_t* vsrc, int32_t* vlen, int32_t* vrow,
     LongRow* lrows) {
-  __shared__ int64_t start[LD_WARPS][LD_MAX_VMAX + 1];  // first sorted position of a length
-  __shared__ int64_t cntl[LD_WARPS][LD_MAX_VMAX + 1];   // pieces of a length
-  __shared__ int64_t pos[LD_WARPS][LD_MAX_VMAX + 1];    // next free position of a length
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t win = (int64_t)blockIdx.x * LD_WARPS + w;
-  if (win >= nwin) return;  // uniform per warp
+  __shared__ WinShared S;
+  __shared__ unsigned pos[LD_WARPS][LD_MAX_VMAX + 1];  // next position of a length in its class
+  struct Big {
+    int64_t lane, first, pid, nf;
+    int32_t row;
+  };
+  __shared__ Big big[LD_BIG];
+  __shared__ int nbig;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int64_t win = blockIdx.x;
   const int64_t at_slices = off[win], at_entries = off[nwin + win];
   const int64_t at_pieces = off[2 * nwin + win], at_lrows = off[3 * nwin + win];
-  for (int l = lane; l <= vmax; l += 32) cntl[w][l] = 0;
-  __syncwarp();
   const int64_t r0 = win * window, r1 = r0 + window < n ? r0 + window : n;
-  for (int64_t r = r0 + lane; r < r1; r += 32) {
-    int64_t nfull;
-    int s;
-    row_pieces(R.L(r), vmax, nfull, s);
-    if (nfull) atomicAdd(reinterpret_cast<unsigned long long*>(&cntl[w][vmax]),
-                         (unsigned long long)nfull);
-    if (s) atomicAdd(reinterpret_cast<unsigned long long*>(&cntl[w][s]), 1ull);
-  }
-  __syncwarp();
-  if (lane == 0) {
-    int64_t acc = 0;
-    for (int L = vmax; L >= 1; --L) {
-      start[w][L] = acc;
-      pos[w][L] = acc;
-      acc += cntl[w][L];
+  int64_t s0, s1;
+  win_share(r0, r1, s0, s1);
+  if (threadIdx.x == 0) nbig = 0;
+  win_classes(R, r0, r1, s0, s1, vmax, S);
+  // the shares before this warp's, class by class
+  for (int l = threadIdx.x; l < vmax; l += blockDim.x) {
+    unsigned run = 0;
+    for (int q = 0; q < nw; ++q) {
+      pos[q][l] = run;
+      run += S.cnt[q][l];
     }
-    start[w][0] = acc;  // the window's pieces
   }
-  __syncwarp();
-  const int64_t np = start[w][0];
+  int64_t pfull = 0, piece_run = at_pieces, lrow_run = at_lrows;
+  for (int q = 0; q < w; ++q) {
+    pfull += S.full[q];
+    piece_run += S.cutp[q];
+    lrow_run += S.cut[q];
+  }
+  const int64_t np = S.np;
   const int64_t nsl = (np + SELL_C - 1) / SELL_C;
   // slices: slice j starts at sorted position 32 j and takes the length of
-  // the piece there; their entries follow one another
-  int64_t ebase = at_entries;
-  for (int64_t j0 = 0; j0 < nsl; j0 += 32) {
-    const int64_t j = j0 + lane;
-    int L = 0;
-    if (j < nsl) {
-      const int64_t p = j * SELL_C;
-      for (int l = vmax; l >= 1; --l)
-        if (cntl[w][l] > 0 && start[w][l] <= p && p < start[w][l] + cntl[w][l]) {
-          L = l;
-          break;
-        }
+  // the piece there (the smallest length whose class starts at or before it:
+  // classes without pieces start where the next shorter one does)
+  for (int64_t j = threadIdx.x; j < nsl; j += blockDim.x) {
+    const int64_t p = j * SELL_C;
+    int lo = 1, hi = vmax;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (S.start[mid] <= p) hi = mid;
+      else lo = mid + 1;
     }
-    int64_t tot;
-    const int64_t ex = warp_excl_scan((int64_t)SELL_C * L, &tot);
-    if (j < nsl) {
-      SellSlice sl;
-      sl.base = ebase + ex;
-      sl.len = L;
-      sl.pad_ = 0;
-      slices[at_slices + j] = sl;
-    }
-    ebase += tot;
+    SellSlice sl;
+    sl.base = at_entries + S.ebase[lo] +
+              (j - (S.start[lo] + SELL_C - 1) / SELL_C) * SELL_C * (int64_t)lo;
+    sl.len = lo;
+    sl.pad_ = 0;
+    slices[at_slices + j] = sl;
   }
+  __syncthreads();
   // pieces, in row order
   const int64_t lane0 = at_slices * SELL_C;
-  int64_t piece_run = at_pieces, lrow_run = at_lrows;
-  for (int64_t c0 = r0; c0 < r1; c0 += 32) {
+  for (int64_t c0 = s0; c0 < s1; c0 += 32) {
     const int64_t r = c0 + lane;
-    const bool ok = r < r1;
+    const bool ok = r < s1;
     const int64_t L = ok ? R.L(r) : 0;
     int64_t nfull;
     int s;
@@ -421,12 +499,11 @@ __global__ void __launch_bounds__(32 * LD_WARPS) win_emit_kernel(
     const int64_t exf = warp_excl_scan(nfull, &tf);
     const int64_t exp_ = warp_excl_scan(npc, &tp);
     const int64_t exl = warp_excl_scan((int64_t)(cut ? 1 : 0), &tl);
-    const int64_t pf = pos[w][vmax] + exf;
-    const int key = s ? s : 0;
-    const unsigned peers = __match_any_sync(0xffffffffu, key);
-    const int64_t bs = s ? pos[w][s] : 0;
+    const int64_t pf = pfull + exf;
+    pfull += tf;
+    const unsigned peers = __match_any_sync(0xffffffffu, s);
+    const unsigned bs = s ? pos[w][s] : 0u;
     __syncwarp();
-    if (lane == 0) pos[w][vmax] += tf;
     if (s && lane == __ffs(peers) - 1) pos[w][s] = bs + __popc(peers);
     __syncwarp();
     const int64_t first = ok && L > 0 ? R.first(r) : 0;
@@ -434,7 +511,7 @@ __global__ void __launch_bounds__(32 * LD_WARPS) win_emit_kernel(
     const int64_t pid = piece_run + exp_;
     // full-length pieces: a row with one writes it; the pieces of a row cut
     // into several are written by the whole warp, row by row (consecutive
-    // lanes, coalesced)
+    // lanes, coalesced), those of a hub row by the whole CTA below
     if (nfull == 1) {
       const int64_t l = lane0 + pf;
       vout[l] = cut ? (int32_t)(-1 - pid) : (int32_t)r;
@@ -442,7 +519,19 @@ __global__ void __launch_bounds__(32 * LD_WARPS) win_emit_kernel(
       vlen[l] = vmax;
       if (vrow) vrow[l] = o;
     }
-    for (unsigned many = __ballot_sync(0xffffffffu, nfull > 1); many; many &= many - 1) {
+    bool mine = nfull > 1;
+    if (nfull > LD_BIG_PIECES) {
+      const int q = atomicAdd(&nbig, 1);
+      if (q < LD_BIG) {
+        big[q].lane = lane0 + pf;
+        big[q].first = first;
+        big[q].pid = pid;
+        big[q].nf = nfull;
+        big[q].row = o;
+        mine = false;
+      }
+    }
+    for (unsigned many = __ballot_sync(0xffffffffu, mine); many; many &= many - 1) {
       const int src_lane = __ffs(many) - 1;
       const int64_t nf = __shfl_sync(0xffffffffu, nfull, src_lane);
       const int64_t pf_l = __shfl_sync(0xffffffffu, pf, src_lane);
@@ -459,7 +548,7 @@ __global__ void __launch_bounds__(32 * LD_WARPS) win_emit_kernel(
     }
     if (ok && L > 0) {
       if (s) {
-        const int64_t l = lane0 + bs + __popc(peers & lanemask_lt());
+        const int64_t l = lane0 + S.start[s] + bs + __popc(peers & lanemask_lt());
         vout[l] = cut ? (int32_t)(-1 - (pid + nfull)) : (int32_t)r;
         vsrc[l] = first + nfull * vmax;
         vlen[l] = s;
@@ -478,11 +567,21 @@ __global__ void __launch_bounds__(32 * LD_WARPS) win_emit_kernel(
     lrow_run += tl;
   }
   // lanes past the last piece of the window's last slice
-  for (int64_t l = lane0 + np + lane; l < lane0 + nsl * SELL_C; l += 32) {
+  for (int64_t l = lane0 + np + threadIdx.x; l < lane0 + nsl * SELL_C; l += blockDim.x) {
     vout[l] = SELL_SKIP;
     vsrc[l] = 0;
     vlen[l] = 0;
     if (vrow) vrow[l] = -1;
+  }
+  __syncthreads();
+  for (int q = 0; q < min(nbig, LD_BIG); ++q) {
+    const Big B = big[q];
+    for (int64_t c = threadIdx.x; c < B.nf; c += blockDim.x) {
+      vout[B.lane + c] = (int32_t)(-1 - (B.pid + c));
+      vsrc[B.lane + c] = B.first + c * vmax;
+      vlen[B.lane + c] = vmax;
+      if (vrow) vrow[B.lane + c] = B.row;
+    }
   }
 }
 
@@ -507,18 +606,6 @@ __global__ void lrow_gather_kernel(const LongRow* in, const int32_t* idx, int64_
   big = warp_isum(big);
   if ((threadIdx.x & 31) == 0 && big) atomicAdd(nbig, big);
 }
-__global__ void lrow_cmax_kernel(const LongRow* lr, int64_t nl, unsigned int* cmax) {
-  unsigned m = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nl;
-       i += (int64_t)gridDim.x * blockDim.x)
-    m = (unsigned)lr[i].count > m ? (unsigned)lr[i].count : m;
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned y = __shfl_down_sync(0xffffffffu, m, o);
-    m = y > m ? y : m;
-  }
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(cmax, m);
-}
-
 int grid_for(int64_t items, int threads, int cap = 16384) {
   int64_t b = (items + threads - 1) / threads;
   if (b < 1) b = 1;
@@ -621,6 +708,7 @@ cudaError_t DevLayout::count(const int64_t* rp_dev, int64_t n_, int64_t nnz_, in
     err = "row_ptr must be non-decreasing";
     return cudaErrorInvalidValue;
   }
+  longest = (int64_t)h.lmax;
   if (reorder) {
     const uint32_t L = (uint32_t)std::min<unsigned long long>(h.lmax, 0xffffffffull);
     flip_keys_kernel<<<grid_for(n, 256), 256, 0, s>>>(k0, n, L);
@@ -645,14 +733,18 @@ cudaError_t DevLayout::order(int32_t* perm, int32_t* iperm, int64_t* src, int32_
 
 cudaError_t DevLayout::windows(cudaStream_t s, int64_t* totals_host) {
   RowsView R{rp, view_src, view_len, view_perm};
-  const unsigned blocks = (unsigned)((nwin + LD_WARPS - 1) / LD_WARPS);
-  win_count_kernel<<<blocks, 32 * LD_WARPS, 0, s>>>(R, n, window, vmax, nwin, wc);
+  win_count_kernel<<<(unsigned)nwin, 32 * ld_warps(window), 0, s>>>(R, n, window, vmax, nwin, wc);
   cudaError_t e = cudaGetLastError();
   int64_t* tmp = wc - (SCAN_MAX_BLOCKS + 1);
   int64_t* tot = reinterpret_cast<int64_t*>(reinterpret_cast<unsigned char*>(wc) +
                                             (size_t)4 * std::max<int64_t>(nwin, 1) * 8 + 16);
-  for (int f = 0; f < 4 && e == cudaSuccess; ++f)
-    e = excl_scan(wc + (size_t)f * nwin, nwin, tmp, tot + f, s);
+  if (e == cudaSuccess && nwin <= SCAN_BLOCK) {  // one block per field
+    scan_one_block_kernel<<<4, SCAN_THREADS, 0, s>>>(wc, nwin, tot);
+    e = cudaGetLastError();
+  } else {
+    for (int f = 0; f < 4 && e == cudaSuccess; ++f)
+      e = excl_scan(wc + (size_t)f * nwin, nwin, tmp, tot + f, s);
+  }
   if (e == cudaSuccess) e = cudaMemcpyAsync(totals_host, tot, 4 * 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) {
@@ -668,9 +760,8 @@ cudaError_t DevLayout::emit(SellSlice* slices, int32_t* vout, int64_t* vsrc, int
                             int32_t* vrow, LongRow* lrows, LongRow* lrows_tmp, cudaStream_t s,
                             int* nbig_host) {
   RowsView R{rp, view_src, view_len, view_perm};
-  const unsigned blocks = (unsigned)((nwin + LD_WARPS - 1) / LD_WARPS);
-  win_emit_kernel<<<blocks, 32 * LD_WARPS, 0, s>>>(R, n, window, vmax, nwin, wc, slices, vout,
-                                                   vsrc, vlen, vrow, lrows_tmp);
+  win_emit_kernel<<<(unsigned)nwin, 32 * ld_warps(window), 0, s>>>(
+      R, n, window, vmax, nwin, wc, slices, vout, vsrc, vlen, vrow, lrows_tmp);
   cudaError_t e = cudaGetLastError();
   *nbig_host = 0;
   if (e != cudaSuccess || nlrows == 0) return e;
@@ -688,17 +779,11 @@ cudaError_t DevLayout::emit(SellSlice* slices, int32_t* vout, int64_t* vsrc, int
   int64_t* tmp = cnt + (size_t)ntiles * DS_BINS;
   unsigned char* tail =
       reinterpret_cast<unsigned char*>(wc + 4 * std::max<int64_t>(nwin, 1)) + 64;
-  unsigned* cmax = reinterpret_cast<unsigned*>(tail);
   int* nbig = reinterpret_cast<int*>(tail + 8);
   e = cudaMemsetAsync(tail, 0, 16, s);
-  if (e == cudaSuccess) {
-    lrow_cmax_kernel<<<grid_for(nlrows, 256), 256, 0, s>>>(lrows_tmp, nlrows, cmax);
-    e = cudaGetLastError();
-  }
-  unsigned hc = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, cmax, 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return e;
+  // the longest row has the most pieces
+  const unsigned hc = (unsigned)std::min<int64_t>((longest + vmax - 1) / vmax, 0x7fffffff);
   lrow_keys_kernel<<<grid_for(nlrows, 256), 256, 0, s>>>(lrows_tmp, nlrows, hc, k0, v0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // the cut rows are at most n: the row-order buffers and counts serve again
