@@ -379,5 +379,16 @@ TE_DEV void bulk_g2s(void* dst_smem, const void* src, uint32_t bytes, uint64_t* 
 TE_DEV void named_bar_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
+// the same, and whether any of the threads brought `pred`
+TE_DEV bool named_bar_or(int id, int threads, bool pred) {
+  int any;
+  asm volatile(
+      "{ .reg .pred p, q;\n setp.ne.b32 p, %3, 0;\n barrier.cta.red.or.pred q, %1, %2, p;\n"
+      " selp.b32 %0, 1, 0, q; }"
+      : "=r"(any)
+      : "r"(id), "r"(threads), "r"((int)pred)
+      : "memory");
+  return any != 0;
+}
 
 }  // namespace te

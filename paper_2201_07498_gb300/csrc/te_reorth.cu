@@ -96,6 +96,19 @@ constexpr int GROUP_MIN_PER_CTA = 8;
 
 __host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// DDD dots of the delayed form (IntDots): the digits of a tile's vectors in
+// binary16, two buffers; a digit's row is 32 bytes longer than the tile, so that
+// the eight digits lie in different banks
+constexpr int DIG_LD = TILE_R + 16;
+__host__ __device__ constexpr bool has_digits(int prec, int mode) {
+  return prec == PREC_DDD && mode == MODE_DCGS_DOT;
+}
+struct __align__(16) DigitBuf {
+  uint16_t d[2][2][8][DIG_LD];    // [buffer][vector][digit][row]
+  int64_t acc[8][CONSUMERS];      // sums of products: [fragment x half][thread]
+  int wmax[CONSUMERS / 32];       // a warp's largest exponent
+  int ecol[MAX_M + 2];            // bound on a column's (biased) exponent
+};
 // DDD updates: a column's small coefficients in binary32 (scaled), and the
 // exponent that brings its elements into binary32's range
 struct __align__(16) LowCoef {
@@ -104,7 +117,8 @@ struct __align__(16) LowCoef {
 };
 
 struct SmemPlan {
-  size_t region, ws_off, coef_off, coef2_off, ritz_off, red_off, fin_off, low_off, bar_off, total;
+  size_t region, ws_off, coef_off, coef2_off, ritz_off, red_off, fin_off, dig_off, low_off, bar_off,
+      total;
 };
 // finalize scratch (doubles): copies of s, alpha, beta, the c_j, warp sums
 constexpr int FIN_SCRATCH = 4 * (MAX_M + 2) + 2 * (CONSUMERS / 32) + 8;
@@ -119,9 +133,10 @@ __host__ __device__ inline SmemPlan smem_plan(int prec, int mode, size_t region,
   size_t ritz = (mode == MODE_RITZ) ? align_up((size_t)ritz_elems * 8, 128) : 0;
   p.red_off = p.ritz_off + ritz;
   p.fin_off = align_up(p.red_off + PSTRIDE * 8, 8);
-  p.low_off = align_up(p.fin_off + FIN_SCRATCH * 8, alignof(LowCoef));
-  p.bar_off = align_up(
-      p.low_off + (prec == PREC_DDD && mode != MODE_RITZ ? sizeof(LowCoef) * MAX_M : 0), 8);
+  const bool ddd = prec == PREC_DDD && mode != MODE_RITZ;
+  p.dig_off = align_up(p.fin_off + FIN_SCRATCH * 8, alignof(DigitBuf));
+  p.low_off = align_up(p.dig_off + (has_digits(prec, mode) ? sizeof(DigitBuf) : 0), alignof(LowCoef));
+  p.bar_off = align_up(p.low_off + (ddd ? sizeof(LowCoef) * MAX_M : 0), 8);
   p.total = p.bar_off + 2 * MAX_STAGES * 8 + 32;
   return p;
 }
@@ -295,6 +310,205 @@ TE_DEV void low_coefs(const PassArgs& a, LowCoef* lc, int* info, int lane) {
     o.bias = (ec - 127) * (1 << 20);  // an element times 2^-(ec - 1023), below 1 in magnitude
     o.pad_ = 0;
     lc[j] = o;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// DDD dots of the delayed form on the tensor pipe
+// ---------------------------------------------------------------------------
+// A warp's binary64 instruction holds its scheduler's unit for 64 cycles, so a
+// pass that takes two dots with every basis element is bound by them far
+// below the memory rate (R-MAT 2^22, 16 columns on average: pass 1 301 us at 25 %
+// of the DRAM peak, the binary64 pipe 77 % busy).  Over enough tiles the dots are
+// therefore taken exactly, in digits (the splitting of Ozaki, Ogita, Oishi &
+// Rump, Numer. Algorithms 59, 2012):
+//   - an element becomes a sign and a fixed-point magnitude X < 2^61, |x| =
+//     X 2^(E - 1083), with E a bound on the biased exponents of its column (the
+//     norm's plus one) or of the vector (the largest seen so far, plus three).
+//     What is cut off lies below 2^-59 of the column's norm (2^-57 of the
+//     vector's largest element), under the rounding of binary64 sums;
+//   - the eight bytes of X are digits.  A byte's bits, read as a binary16
+//     number, are that many units of 2^-24 (subnormal, exact), so the basis'
+//     digits need no conversion: bytes with X's sign.  The vectors' are balanced,
+//     -128 ... 128, which binary16 holds exactly too.  mma.sync m16n8k16
+//     multiplies the eight digits of both vectors (16 rows of A) with digit i of
+//     eight columns over 16 tile rows;
+//   - products stay below 2^15 and INT_ROWS = 256 rows of them below 2^23 units:
+//     binary32 accumulators hold the sums exactly, and then pass them on to
+//     64-bit integers (room for 2^23 rows); those go to binary64 at the end, or
+//     when the vector's bound grows.
+// Infinities and NaN have no digits: the dots of a vector or column that holds one
+// are NaN.  Bound by instruction issue and latency, not by the tensor pipe
+// (2^21 rows x 14 columns: ALU 49 % busy, tensor 14 %, DRAM 30 %); two warps per
+// scheduler have registers for it, twice the warps at 96 registers were slower
+// (the pass over 2^22 rows 227 -> 256 us).  With eight-bit integer mma.sync the
+// digits need fewer instructions, but m16n8k32 takes 65 cycles per scheduler on
+// this GPU, against 8 for binary16 m16n8k16: 328 us.  Only the delayed form's
+// pass takes two dots per element; with one, digits were slower (Lanczos phase,
+// 524,287 rows, m 40: 8.55 ms against 8.35).
+constexpr int INT_ROWS = 256;
+// From this many tiles per CTA and columns on; below, the vectors' digits and the
+// way back to binary64 cost more than the binary64 instructions saved.  32 passes
+// over 0 ... 31 columns, binary64 dots and digits: 2^22 rows 9.64 and 7.26 ms, 2^20
+// (27 tiles per CTA) 2.99 and 2.49, 2^18 (6.7) 1.35 and 1.30; 150,001 rows (3.9)
+// 1.12 and about 1.15.  From 7, 9 or 13 columns on, 2^20 rows: 2.49, 2.50, 2.52.
+constexpr int IDOT_TILES = 6, IDOT_COLS = 8;
+
+// the bound on the exponents of a column with scale s (1 / norm): |x| <= norm,
+// and a binade for the rounding of the norm.  At least 70, so that zeros and
+// subnormals (exponent 0) shift out entirely.
+TE_DEV int digit_exp(double s) { return max(min(column_exp(s) + 1, 2046), 70); }
+// X of |x| for the bound e; what is cut off is jammed into the last bit (its error
+// then has no sign of its own, where a truncation's would add up)
+TE_DEV uint64_t fixed64(double x, int e) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned s = (unsigned)(e - ((hi >> 20) & 0x7ff));
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const uint64_t m = (uint64_t)__funnelshift_l(lo, mh, 8) << 32 | (lo << 8);
+  return m >> min(s, 63u) | (uint64_t)(s - 9u < 52u ? 1u : 0u);
+}
+
+TE_DEV double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }  // (normal)
+
+TE_DEV void mma_f16(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
+                    unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// The dots of up to 8 DIG_W = MAX_M basis columns with the two vectors.  Columns go in groups of
+// 8; a group's warps share the 16-row steps of every tile.
+constexpr int DIG_W = CONSUMERS / 32;
+static_assert(8 * DIG_W >= MAX_M, "a warp takes one group");
+struct DigShare {  // group q's warps: [w0, w1)
+  int w0, w1;
+  TE_DEV DigShare(int ncols, int q) {
+    const int groups = (ncols + 7) / 8;  // <= DIG_W
+    w0 = (q * DIG_W + groups - 1) / groups;
+    w1 = ((q + 1) * DIG_W + groups - 1) / groups;
+  }
+};
+struct IntDots {
+  float acc[8][4];       // [basis digit]: vector digit g of each vector x columns 2 t, 2 t + 1
+  int64_t* wide;         // the same, emptied into shared memory: [fragment][half][thread]
+  double sum[4];         // [vector][columns 2 t, 2 t + 1] (lanes with g = 0)
+  int ncols, group, first, count, rows;  // this warp's columns, steps, rows in acc
+  int ec, ev[2];        // exponent bounds of column g and of the vectors
+
+  TE_DEV void init(int ncols_, const int* ecol, int64_t* wide_, int wid, int lane) {
+    ncols = ncols_;
+    wide = wide_;
+    rows = 0;
+    const int groups = (ncols + 7) / 8;
+    group = wid * groups / DIG_W;
+    const DigShare sh(ncols, group);
+    constexpr int STEPS = TILE_R / 16;
+    first = STEPS * (wid - sh.w0) / (sh.w1 - sh.w0);
+    count = STEPS * (wid - sh.w0 + 1) / (sh.w1 - sh.w0) - first;
+    const int c = 8 * group + (lane >> 2);
+    ec = c < ncols ? max(ecol[c], 70) : 2046;
+#pragma unroll
+    for (int v = 0; v < 2; ++v) ev[v] = 70;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      sum[c] = 0.0;
+      wide[2 * c * CONSUMERS] = wide[(2 * c + 1) * CONSUMERS] = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i][c] = 0.f;
+    }
+  }
+  // the accumulators (integers up to 2^23, in units of 2^-24) into `wide`: basis
+  // digits 0 ... 3 and 4 ... 7
+  TE_DEV void empty() {
+    rows = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        int64_t y = wide[(2 * c + h) * CONSUMERS];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          y += (int64_t)__float2int_rn(acc[4 * h + i][c] * 0x1p24f) * (1 << (8 * i));
+          acc[4 * h + i][c] = 0.f;
+        }
+        wide[(2 * c + h) * CONSUMERS] = y;
+      }
+  }
+  // everything so far into binary64 (a fixed order)
+  TE_DEV void flush(int lane) {
+    empty();
+    const int g = lane >> 2, t = lane & 3;
+    const double scale = pow2(8 * g);  // 256^g
+    const int e0 = __shfl_sync(0xffffffffu, ec, 8 * t), e1 = __shfl_sync(0xffffffffu, ec, 8 * t + 4);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      int64_t* o = wide + 2 * c * CONSUMERS;
+      double d = fma((double)o[CONSUMERS], 4294967296.0, (double)o[0]) * scale;
+      o[0] = o[CONSUMERS] = 0;
+#pragma unroll
+      for (int x = 4; x < 32; x *= 2) d += __shfl_xor_sync(0xffffffffu, d, x);
+      // (two factors: either alone may leave binary64's range)
+      sum[c] += d * pow2((c & 1 ? e1 : e0) - 1083) * pow2(ev[c / 2] - 1083);
+    }
+  }
+  // one tile: the basis columns at tv, the vectors' digits
+  TE_DEV void tile(const double* tv, const uint16_t (*dig)[8][DIG_LD], int lane) {
+    const int g = lane >> 2, t = lane & 3;
+    const int c = 8 * group + g;
+    const double* col = tv + (size_t)c * TILE_R + 4 * t;
+    const bool mine = c < ncols;
+#pragma unroll 2
+    for (int k = first; k < first + count; ++k) {
+      const int r0 = 16 * k;  // this lane's rows r0 + 4 t ... r0 + 4 t + 3
+      double2 x0 = make_double2(0.0, 0.0), x1 = x0;
+      if (mine) {
+        x0 = *reinterpret_cast<const double2*>(col + r0);
+        x1 = *reinterpret_cast<const double2*>(col + r0 + 2);
+      }
+      unsigned b[8][2];  // [digit][two rows in the halves of a register]
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const double xa = u ? x1.x : x0.x, xb = u ? x1.y : x0.y;
+        const uint64_t za = fixed64(xa, ec), zb = fixed64(xb, ec);
+        const unsigned sg = __byte_perm((unsigned)__double2hiint(xa), (unsigned)__double2hiint(xb),
+                                        0x7030) & 0x80008000u;
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+          const unsigned ya = (unsigned)(za >> (32 * w)), yb = (unsigned)(zb >> (32 * w));
+          const unsigned p = __byte_perm(ya, yb, 0x5410), q = __byte_perm(ya, yb, 0x7632);
+          b[4 * w][u] = (p & 0x00ff00ffu) | sg;
+          b[4 * w + 1][u] = ((p >> 8) & 0x00ff00ffu) | sg;
+          b[4 * w + 2][u] = (q & 0x00ff00ffu) | sg;
+          b[4 * w + 3][u] = ((q >> 8) & 0x00ff00ffu) | sg;
+        }
+      }
+      const uint2 a0 = *reinterpret_cast<const uint2*>(&dig[0][g][r0 + 4 * t]);
+      const uint2 a1 = *reinterpret_cast<const uint2*>(&dig[1][g][r0 + 4 * t]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) mma_f16(acc[i], a0.x, a1.x, a0.y, a1.y, b[i][0], b[i][1]);
+    }
+    rows += 16 * count;
+    if (rows + 16 * count > INT_ROWS) empty();
+  }
+};
+
+// the eight balanced digits of x (bound e) for row r: byte j of X + 0x80...80 as
+// 1024 + byte in binary16, then less 1152 and with x's sign
+TE_DEV void put_digits(uint16_t (*dig)[DIG_LD], int r, double x, int e) {
+  const uint64_t z = fixed64(x, e) + 0x8080808080808080ull;
+  const unsigned sg = ((unsigned)__double2hiint(x) & 0x80000000u) | ((unsigned)__double2hiint(x) >> 16 & 0x8000u);
+  const unsigned one = 0x3c003c00u ^ sg, off = 0xe480e480u ^ sg;  // +-1, -+1152
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    const unsigned w = (unsigned)(z >> (j < 4 ? 0 : 32));
+    const unsigned p = __byte_perm(w, 0x64646464u, j & 2 ? 0x4342 : 0x4140);
+    unsigned d;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(p), "r"(one), "r"(off));
+    dig[j][r] = (uint16_t)d;
+    dig[j + 1][r] = (uint16_t)(d >> 16);
   }
 }
 
@@ -497,7 +711,8 @@ TE_DEV void finalize_pass(const PassArgs& a, const double* tot, double* scr, con
 // One CTA's share of a pass: CTA `cta` of `ncta` takes tiles cta, cta + ncta, ...
 // (the single-solve kernel passes blockIdx.x / gridDim.x; the batched kernel
 // of the serving engine maps its blocks onto the CTAs of several solves).
-template <int P, int MODE>
+// DIG: DDD dots in digits.
+template <int P, int MODE, bool DIG = false>
 __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, const int cta,
                                           const int ncta) {
   using Tr = PassTr<P>;
@@ -583,6 +798,17 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
     for (int j = tid; j < nb - 1; j += PASS_THREADS) {
       coef[j] = to_coef<P>(st->c1[j]);
       coef2[j] = to_coef<P>(st->c2[j]);
+    }
+  }
+  // dots in digits, over the columns before the candidate
+  static_assert(!DIG || has_digits(P, MODE), "");
+  DigitBuf* dig = reinterpret_cast<DigitBuf*>(sm + L.dig_off);
+  const int idcols = nb - 1;
+  bool poisoned = false;  // the pass vector holds an infinity or NaN
+  if constexpr (DIG) {
+    for (int j = tid; j < nb; j += PASS_THREADS) {
+      const double sj = st->s[a.col0 + j];
+      dig->ecol[j] = sj > 0.0 && biased_exp(sj) < 0x7ff ? digit_exp(sj) : -1;  // (no finite norm)
     }
   }
   LowCoef* lowc = reinterpret_cast<LowCoef*>(sm + L.low_off);
@@ -672,6 +898,35 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
 #pragma unroll
   for (int q = 0; q < (DDOT ? QMAX : 1); ++q) dots2[q] = zero_acc<P>();
   const bool low = P == PREC_DDD && (HAS_AXPY || DUPD) && lowinfo[0] != 0;
+  IntDots idots{};
+  int idbuf = 0;
+  bool started = false;
+  if constexpr (DIG) {
+    idots.init(idcols, dig->ecol, &dig->acc[0][tid], wid, lane);
+    idots.ev[1] = max(dig->ecol[nb - 1], 70);
+  }
+  // a tile's digits of the vector x (and the candidate's element sc), then its
+  // dots; every consumer thread, with its row's values
+  auto int_tile = [&](const double* tv, double x, double sc) {
+    const int e = biased_exp(x);
+    put_digits(dig->d[idbuf][1], tid, sc, idots.ev[1]);
+    put_digits(dig->d[idbuf][0], tid, x, idots.ev[0]);
+    if (named_bar_or(1, CONSUMERS, e > idots.ev[0])) {  // the bound has to grow
+      const int we = __reduce_max_sync(0xffffffffu, e);
+      if (lane == 0) dig->wmax[wid] = we;
+      named_bar_sync(1, CONSUMERS);
+      int tm = 0;
+      for (int w = 0; w < CONSUMERS / 32; ++w) tm = max(tm, dig->wmax[w]);
+      if (tm == 0x7ff) poisoned = true;
+      if (started) idots.flush(lane);
+      idots.ev[0] = min(tm + 3, 2047);
+      put_digits(dig->d[idbuf][0], tid, x, idots.ev[0]);
+      named_bar_sync(1, CONSUMERS);
+    }
+    idots.tile(tv, dig->d[idbuf], lane);
+    started = true;
+    idbuf ^= 1;
+  };
   acc_t n1 = zero_acc<P>(), n2 = zero_acc<P>();
   basis_t* Vout = static_cast<basis_t*>(a.Vmut) + (size_t)a.col_out * a.cstride;
 
@@ -798,7 +1053,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
             n1 = fma(w, w, n1);
           }
         }
-      } else if constexpr (MODE == MODE_DOT || DDOT) {
+      } else if constexpr (!DIG && (MODE == MODE_DOT || DDOT)) {
         ws[tid] = x;
       }
       if constexpr (DDOT) {
@@ -811,6 +1066,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
         } else {
           n1 = fma(sc, x, n1);
           n2 = fma(sc, sc, n2);
+          if constexpr (DIG) int_tile(tv, x, sc);
         }
       }
 
@@ -896,7 +1152,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
         }
       }
 
-      if constexpr (DDOT) {
+      if constexpr (DDOT && !DIG) {
         named_bar_sync(1, CONSUMERS);
         // delayed reorthogonalisation, warp per column: the dot of every column
         // with y (the first sweep of the new vector) and with the candidate
@@ -1087,7 +1343,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
         }
       }
 
-      if constexpr (HAS_DOT || DDOT) named_bar_sync(1, CONSUMERS);
+      if constexpr (HAS_DOT || (DDOT && !DIG)) named_bar_sync(1, CONSUMERS);
     }  // tiles of the group
     if (nb > 0) {
       __syncwarp();
@@ -1098,6 +1354,28 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
   if (a.fin == FIN_NONE) return;
 
   // ---- per-CTA partial sums ----
+  if constexpr (DIG) {  // the warps' shares of a column, added in warp order
+    idots.flush(lane);
+    double* part = reinterpret_cast<double*>(dig->d);  // [warp][vector][8]
+    named_bar_sync(1, CONSUMERS);                      // (its digits have been read)
+    if (lane < 4) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        part[(wid * 2 + c / 2) * 8 + 2 * lane + (c & 1)] = idots.sum[c];
+    }
+    named_bar_sync(1, CONSUMERS);
+    if (tid < idcols) {
+      const DigShare sh(idcols, tid / 8);
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        double t = 0.0;
+        for (int w = sh.w0; w < sh.w1; ++w) t += part[(w * 2 + v) * 8 + (tid & 7)];
+        if ((v ? dig->ecol[nb - 1] < 0 : poisoned) || dig->ecol[tid] < 0)
+          t = __longlong_as_double(0x7ff8000000000000ll);
+        put_partial<P>(a.partials, pidx(v ? SLOT_D2 + tid : tid, cta, ncta), t);
+      }
+    }
+  }
   if constexpr (HAS_DOT) {
     const int jend = (MODE == MODE_AXPY_DOT && P == PREC_FDF) ? nb - 1 : nb;
 #pragma unroll
@@ -1111,7 +1389,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
       }
     }
   }
-  if constexpr (DDOT) {
+  if constexpr (DDOT && !DIG) {
 #pragma unroll
     for (int q = 0; q < QMAX; ++q) {
       const int jj = wid + (CONSUMERS / 32) * q;
@@ -1199,9 +1477,9 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
   }
 }
 
-template <int P, int MODE>
+template <int P, int MODE, bool DIG = false>
 __global__ void __launch_bounds__(PASS_THREADS, pass_ctas_per_sm(P)) pass_kernel(PassArgs a, size_t region) {
-  pass_body<P, MODE>(a, region, (int)blockIdx.x, (int)gridDim.x);
+  pass_body<P, MODE, DIG>(a, region, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1334,6 +1612,11 @@ static cudaError_t config_t(int max_cols, int K, int num_sms, PassLaunch& out) {
   e = cudaFuncSetAttribute(pass_kernel<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)total);
   if (e != cudaSuccess) return e;
+  if constexpr (has_digits(P, MODE)) {
+    e = cudaFuncSetAttribute(pass_kernel<P, MODE, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)total);
+    if (e != cudaSuccess) return e;
+  }
   out.grid = num_sms * pass_ctas_per_sm(P);
   out.smem = total;
   out.stages = stages;
@@ -1364,7 +1647,14 @@ cudaError_t launch_pass(int prec, int mode, const PassArgs& a, const PassLaunch&
                         cudaStream_t s) {
 #define TE_LAUNCH(PP, MM)                                                        \
   if (prec == PP && mode == MM) {                                                \
-    pass_kernel<PP, MM><<<L.grid, PASS_THREADS, L.smem, s>>>(a, L.region);       \
+    bool dig = false;                                                            \
+    if constexpr (has_digits(PP, MM))                                            \
+      dig = a.nb - 1 >= IDOT_COLS && a.ld / TILE_R >= (int64_t)IDOT_TILES * L.grid; \
+    if (dig)                                                                     \
+      pass_kernel<PP, MM, has_digits(PP, MM)>                                    \
+          <<<L.grid, PASS_THREADS, L.smem, s>>>(a, L.region);                    \
+    else                                                                         \
+      pass_kernel<PP, MM><<<L.grid, PASS_THREADS, L.smem, s>>>(a, L.region);     \
     return cudaGetLastError();                                                   \
   }
   TE_LAUNCH(PREC_DDD, MODE_DOT)
