@@ -379,6 +379,22 @@ TE_DEV void mma_f16(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsign
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// the bytes of two elements (bounds ea, eb) with their signs: b[digit][u]
+TE_DEV void byte_digits(double xa, int ea, double xb, int eb, unsigned (&b)[8][2], int u) {
+  const uint64_t za = fixed64(xa, ea), zb = fixed64(xb, eb);
+  const unsigned sg = __byte_perm((unsigned)__double2hiint(xa), (unsigned)__double2hiint(xb),
+                                  0x7030) & 0x80008000u;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const unsigned ya = (unsigned)(za >> (32 * w)), yb = (unsigned)(zb >> (32 * w));
+    const unsigned p = __byte_perm(ya, yb, 0x5410), q = __byte_perm(ya, yb, 0x7632);
+    b[4 * w][u] = (p & 0x00ff00ffu) | sg;
+    b[4 * w + 1][u] = ((p >> 8) & 0x00ff00ffu) | sg;
+    b[4 * w + 2][u] = (q & 0x00ff00ffu) | sg;
+    b[4 * w + 3][u] = ((q >> 8) & 0x00ff00ffu) | sg;
+  }
+}
+
 // The dots of up to 8 DIG_W = MAX_M basis columns with the two vectors.  Columns go in groups of
 // 8; a group's warps share the 16-row steps of every tile.
 constexpr int DIG_W = CONSUMERS / 32;
@@ -469,22 +485,8 @@ struct IntDots {
         x1 = *reinterpret_cast<const double2*>(col + r0 + 2);
       }
       unsigned b[8][2];  // [digit][two rows in the halves of a register]
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const double xa = u ? x1.x : x0.x, xb = u ? x1.y : x0.y;
-        const uint64_t za = fixed64(xa, ec), zb = fixed64(xb, ec);
-        const unsigned sg = __byte_perm((unsigned)__double2hiint(xa), (unsigned)__double2hiint(xb),
-                                        0x7030) & 0x80008000u;
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-          const unsigned ya = (unsigned)(za >> (32 * w)), yb = (unsigned)(zb >> (32 * w));
-          const unsigned p = __byte_perm(ya, yb, 0x5410), q = __byte_perm(ya, yb, 0x7632);
-          b[4 * w][u] = (p & 0x00ff00ffu) | sg;
-          b[4 * w + 1][u] = ((p >> 8) & 0x00ff00ffu) | sg;
-          b[4 * w + 2][u] = (q & 0x00ff00ffu) | sg;
-          b[4 * w + 3][u] = ((q >> 8) & 0x00ff00ffu) | sg;
-        }
-      }
+      byte_digits(x0.x, ec, x0.y, ec, b, 0);
+      byte_digits(x1.x, ec, x1.y, ec, b, 1);
       const uint2 a0 = *reinterpret_cast<const uint2*>(&dig[0][g][r0 + 4 * t]);
       const uint2 a1 = *reinterpret_cast<const uint2*>(&dig[1][g][r0 + 4 * t]);
 #pragma unroll
@@ -495,20 +497,27 @@ struct IntDots {
   }
 };
 
-// the eight balanced digits of x (bound e) for row r: byte j of X + 0x80...80 as
-// 1024 + byte in binary16, then less 1152 and with x's sign
-TE_DEV void put_digits(uint16_t (*dig)[DIG_LD], int r, double x, int e) {
+// the eight balanced digits of x (bound e): byte j of X + 0x80...80 as 1024 + byte
+// in binary16, then less 1152 and with x's sign
+TE_DEV void digits_f16(double x, int e, unsigned (&d)[4]) {  // digits 2 j, 2 j + 1
   const uint64_t z = fixed64(x, e) + 0x8080808080808080ull;
-  const unsigned sg = ((unsigned)__double2hiint(x) & 0x80000000u) | ((unsigned)__double2hiint(x) >> 16 & 0x8000u);
+  const unsigned hi = (unsigned)__double2hiint(x);
+  const unsigned sg = (hi & 0x80000000u) | (hi >> 16 & 0x8000u);
   const unsigned one = 0x3c003c00u ^ sg, off = 0xe480e480u ^ sg;  // +-1, -+1152
 #pragma unroll
-  for (int j = 0; j < 8; j += 2) {
-    const unsigned w = (unsigned)(z >> (j < 4 ? 0 : 32));
-    const unsigned p = __byte_perm(w, 0x64646464u, j & 2 ? 0x4342 : 0x4140);
-    unsigned d;
-    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(p), "r"(one), "r"(off));
-    dig[j][r] = (uint16_t)d;
-    dig[j + 1][r] = (uint16_t)(d >> 16);
+  for (int j = 0; j < 4; ++j) {
+    const unsigned w = (unsigned)(z >> (j < 2 ? 0 : 32));
+    const unsigned p = __byte_perm(w, 0x64646464u, j & 1 ? 0x4342 : 0x4140);
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d[j]) : "r"(p), "r"(one), "r"(off));
+  }
+}
+TE_DEV void put_digits(uint16_t (*dig)[DIG_LD], int r, double x, int e) {
+  unsigned d[4];
+  digits_f16(x, e, d);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    dig[2 * j][r] = (uint16_t)d[j];
+    dig[2 * j + 1][r] = (uint16_t)(d[j] >> 16);
   }
 }
 
@@ -1579,6 +1588,204 @@ cudaError_t launch_batch_pass(int mode, const BatchTable* T, int restart, const 
 }
 
 // ---------------------------------------------------------------------------
+// DDD Ritz vectors on the tensor pipe
+// ---------------------------------------------------------------------------
+// U = V C takes m K binary64 multiply-adds per row, 64 cycles per warp
+// instruction (R-MAT 2^22, m 32, K 16: 3.75 ms, of which 3.5 are those).  In
+// digits as above: element (r, j) of the basis is bounded by row r's largest
+// element (each relative to its column's norm), C's element (j, k) by output k's
+// largest, so both bounds leave the sum over j.  A = sixteen outputs' digit j by
+// sixteen columns, from shared memory in fragment order; B = sixteen columns' digit
+// i by eight rows, from registers.  The products with i + j = s share one
+// accumulator: with s from 6 to 14 what is left out lies below 2^-59 of the
+// product of the two bounds; at most 8 pairs x 64 columns x 2^15 = 2^24 units,
+// exact in binary32.  A row's sums go through 128-bit integers to binary64 with
+// one rounding, by integer instructions.  A row with an infinity or NaN, and
+// coefficients or norms that are not finite or far from 1 (2^-823 ... 2^877), take
+// binary64 multiply-adds.
+// R-MAT 2^22, m 32, K 16, with the gather back to the caller's order: 3.75 -> 0.99
+// ms; 2^20 rows, m 64, K 64: 6.95 -> 1.11.  Against extended precision the vectors'
+// error falls from 2.0e-16 to 0.8e-16 (norm), from 8.6e-16 to 2.0e-16 of |V| |C|
+// (largest element; 200,001 rows, m 32, K 16).
+constexpr int RD_THREADS = 256;
+constexpr int RD_S0 = 6, RD_S = 9;  // accumulators: s - RD_S0
+
+// S 2^T, rounded to nearest
+TE_DEV double int128_scaled(__int128 S, int T) {
+  const bool neg = S < 0;
+  const unsigned __int128 u = neg ? -(unsigned __int128)S : (unsigned __int128)S;
+  const uint64_t uh = (uint64_t)(u >> 64), ul = (uint64_t)u;
+  if ((uh | ul) == 0) return 0.0;
+  const int lz = uh ? __clzll((long long)uh) : 64 + __clzll((long long)ul);
+  const uint64_t top = (uint64_t)((u << lz) >> 64);  // (bits below 2^-63 of it are cut off)
+  const int e = 1023 + 127 - lz + T;
+  if (e > 0 && e < 2046) {
+    const uint64_t bits = (top >> 11) + ((top >> 10) & 1) + ((uint64_t)(e - 1) << 52);
+    return __longlong_as_double((int64_t)(bits | (uint64_t)neg << 63));
+  }
+  const int t = T + 64 - lz;  // top 2^t leaves the normal range
+  const double d = (double)top * pow2(t / 2) * pow2(t - t / 2);
+  return neg ? -d : d;
+}
+
+template <int KS>  // steps of sixteen columns
+__global__ void __launch_bounds__(RD_THREADS, 2) ritz_digits_kernel(PassArgs a) {
+  extern __shared__ __align__(16) uint4 rd_frag[];  // [output tile][step][digit][lane]
+  __shared__ __align__(16) int ec[16 * KS];
+  __shared__ int fk[MAX_M], special;
+  LzState* st = a.st;
+  if (st->eigvecs == nullptr) return;  // uniform: no vectors requested
+  const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int m = a.nb, K = a.K, ot = (K + 15) / 16;
+  const double* C = st->C;
+  if (tid == 0) special = 0;
+  if (tid < 16 * KS) ec[tid] = tid < m ? column_exp(st->s[a.col0 + tid]) : 1023;
+  __syncthreads();
+  int emin = 4096, emax = 0;
+  for (int j = 0; j < 16 * KS; ++j) {
+    emin = min(emin, ec[j]);
+    emax = max(emax, ec[j]);
+  }
+  if (tid == 0 && (emin < 200 || emax > 1900)) special = 1;
+  if (tid < MAX_M) {
+    int f = 70 + emax;
+    for (int j = 0; tid < K && j < m; ++j) {
+      const int b = biased_exp(C[j * K + tid]);
+      if (b == 0x7ff) special = 1;
+      f = max(f, b + ec[j]);
+    }
+    fk[tid] = f;
+  }
+  __syncthreads();
+  for (int i = tid; i < ot * KS * 32; i += RD_THREADS) {
+    const int l = i & 31, ks = (i >> 5) % KS, o = (i >> 5) / KS;
+    unsigned d[2][4][4];  // [output g, g + 8][column][digit pair]
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int j = 16 * ks + 4 * (l & 3) + c, k = 16 * o + 8 * h + (l >> 2);
+        const bool in = j < m && k < K;
+        digits_f16(in ? C[j * K + k] : 0.0, in ? fk[k] - ec[j] : 1023, d[h][c]);
+      }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const unsigned sel = q & 1 ? 0x7632 : 0x5410;
+      rd_frag[((o * KS + ks) * 8 + q) * 32 + l] =
+          make_uint4(__byte_perm(d[0][0][q / 2], d[0][1][q / 2], sel),
+                     __byte_perm(d[1][0][q / 2], d[1][1][q / 2], sel),
+                     __byte_perm(d[0][2][q / 2], d[0][3][q / 2], sel),
+                     __byte_perm(d[1][2][q / 2], d[1][3][q / 2], sel));
+    }
+  }
+  __syncthreads();
+
+  const double* V = static_cast<const double*>(a.V) + (size_t)a.col0 * a.cstride;
+  double* U = st->eigvecs;
+  const int Kr = (K + 1) & ~1, kout = a.urows ? Kr : K;
+  const int64_t blocks = (a.n + 7) / 8;
+  const int64_t warps = (int64_t)gridDim.x * (RD_THREADS / 32);
+  for (int64_t blk = (int64_t)blockIdx.x * (RD_THREADS / 32) + (tid >> 5); blk < blocks; blk += warps) {
+    const int64_t row0 = 8 * blk;
+    const double* src = V + row0 / TILE_R * a.tstride + row0 % TILE_R;
+    double x[KS][4];  // row g: columns 16 ks + 4 t ... + 3
+    int er = 70 - emin, top = 0;
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int j = 16 * ks + 4 * t + c;
+        x[ks][c] = j < m ? src[(size_t)j * a.cstride + g] : 0.0;
+      }
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int b = biased_exp(x[ks][c]);
+        er = max(er, b - ec[16 * ks + 4 * t + c]);
+        top = max(top, b);
+      }
+    er = max(er, __shfl_xor_sync(0xffffffffu, er, 1));
+    er = max(er, __shfl_xor_sync(0xffffffffu, er, 2));
+    const bool slow = special || __any_sync(0xffffffffu, top == 0x7ff);
+    const int e0 = __shfl_sync(0xffffffffu, er, 8 * t), e1 = __shfl_sync(0xffffffffu, er, 8 * t + 4);
+    for (int o = 0; o < ot; ++o) {
+      double out[4];  // outputs g, g + 8 x rows 2 t, 2 t + 1
+      if (slow) {
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          const int k = 16 * o + g + 8 * (q >> 1);
+          double d = 0.0;
+          for (int j = 0; k < K && j < m; ++j)
+            d = fma(src[(size_t)j * a.cstride + 2 * t + (q & 1)], C[j * K + k], d);
+          if (q == 0) out[0] = d;
+          else if (q == 1) out[1] = d;
+          else if (q == 2) out[2] = d;
+          else out[3] = d;
+        }
+      } else {
+        float acc[RD_S][4];
+#pragma unroll
+        for (int q = 0; q < RD_S; ++q)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[q][c] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          const int4 e = *reinterpret_cast<const int4*>(&ec[16 * ks + 4 * t]);
+          unsigned b[8][2];
+          byte_digits(x[ks][0], er + e.x, x[ks][1], er + e.y, b, 0);
+          byte_digits(x[ks][2], er + e.z, x[ks][3], er + e.w, b, 1);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint4 f = rd_frag[((o * KS + ks) * 8 + j) * 32 + lane];
+#pragma unroll
+            for (int i = RD_S0 - j > 0 ? RD_S0 - j : 0; i < 8; ++i)
+              mma_f16(acc[i + j - RD_S0], f.x, f.y, f.z, f.w, b[i][0], b[i][1]);
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          int64_t lo = 0, hi = 0;
+#pragma unroll
+          for (int q = 0; q < RD_S; ++q) {
+            const int v = __float2int_rn(acc[q][c] * 0x1p24f);
+            if (q < 4) lo += (int64_t)v * (1 << (8 * q));
+            else hi += (int64_t)v * ((int64_t)1 << (8 * (q - 4)));
+          }
+          out[c] = int128_scaled(((__int128)hi << 32) + lo,
+                                 (c & 1 ? e1 : e0) + fk[16 * o + g + 8 * (c >> 1)] - 2166 + 8 * RD_S0);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int k = 16 * o + g + 8 * (c >> 1);
+        const int64_t row = row0 + 2 * t + (c & 1);
+        if (k < kout && row < a.n) {
+          if (a.urows) a.urows[(size_t)row * Kr + k] = out[c];
+          else U[(size_t)k * a.n + row] = out[c];
+        }
+      }
+    }
+  }
+}
+
+static size_t ritz_digits_smem(int m, int K) {
+  return (size_t)((K + 15) / 16) * ((m + 15) / 16) * 8 * 32 * sizeof(uint4);
+}
+using RitzDigitsFn = void (*)(PassArgs);
+static RitzDigitsFn ritz_digits_fn(int m) {
+  return m <= 16 ? ritz_digits_kernel<1> : m <= 32 ? ritz_digits_kernel<2>
+       : m <= 48 ? ritz_digits_kernel<3> : ritz_digits_kernel<4>;
+}
+// From m K' = 80 on (K' = K rounded up as the binary64 form pads it): 2^20 rows,
+// binary64 form and digits, K = 1 ... 8: m 4 70 and 131 us, m 8 125 and 135, m 16
+// 240 and 143; 10,000 rows, m 16: 14 and 10 us.
+constexpr int RITZ_DIGITS_MIN = 80;
+static bool ritz_digits(int m, int K) {
+  return m * ((K + RITZ_KC - 1) / RITZ_KC * RITZ_KC) >= RITZ_DIGITS_MIN;
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 template <int P, int MODE>
@@ -1617,6 +1824,11 @@ static cudaError_t config_t(int max_cols, int K, int num_sms, PassLaunch& out) {
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)total);
     if (e != cudaSuccess) return e;
   }
+  if constexpr (P == PREC_DDD && MODE == MODE_RITZ) {
+    e = cudaFuncSetAttribute(ritz_digits_fn(max_cols), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)ritz_digits_smem(max_cols, max_cols));
+    if (e != cudaSuccess) return e;
+  }
   out.grid = num_sms * pass_ctas_per_sm(P);
   out.smem = total;
   out.stages = stages;
@@ -1645,6 +1857,12 @@ cudaError_t pass_config(int prec, int mode, int max_cols, int K, int num_sms, Pa
 
 cudaError_t launch_pass(int prec, int mode, const PassArgs& a, const PassLaunch& L,
                         cudaStream_t s) {
+  if (prec == PREC_DDD && mode == MODE_RITZ && ritz_digits(a.nb, a.K)) {
+    const int64_t blocks = (a.n + 63) / 64;  // of eight warps with eight rows each
+    const int grid = (int)(blocks < 2 * L.grid ? (blocks > 0 ? blocks : 1) : 2 * L.grid);
+    ritz_digits_fn(a.nb)<<<grid, RD_THREADS, ritz_digits_smem(a.nb, a.K), s>>>(a);
+    return cudaGetLastError();
+  }
 #define TE_LAUNCH(PP, MM)                                                        \
   if (prec == PP && mode == MM) {                                                \
     bool dig = false;                                                            \
