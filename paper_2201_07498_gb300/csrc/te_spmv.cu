@@ -186,7 +186,14 @@ constexpr int SPMV_WPB = 8;     // warps (slices) per CTA
 // with rows relabelled by degree, the first HOT_BYTES of x (the most
 // connected columns) are the ones L1 keeps
 constexpr int64_t HOT_BYTES = 128 << 10;
-constexpr int SPMV_UNROLL = 8;  // entries per lane in flight
+// Entries per lane in flight, and the CTAs per SM that the registers are held to:
+// the gathers' latency is hidden better by more warps than by more loads per warp
+// (unless registers spill).  R-MAT 2^22, 128 M entries, rows by degree, us per SpMV
+// with 8 entries and free registers / 4 and free / 4 and 6 CTAs / 4 and 8 CTAs: DDD
+// 431 / 395 / 375 / 415, FDF 291 / 296 / 295 / 286, 8DF 313 / 296 / 296 / 282.  The
+// order of a row's sum does not depend on it (entries alternate between two chains).
+constexpr int SPMV_UNROLL = 4;
+constexpr int spmv_ctas_per_sm(int prec) { return prec == PREC_DDD ? 6 : 8; }
 
 // stored matrix value type per te_dtype, and its streaming load + exact
 // conversion to the arithmetic's input type
@@ -266,7 +273,8 @@ __device__ __forceinline__ void spmv_slice(const SpmvArgs& a, const int slice, c
         if constexpr (sizeof(x_t) == 4)
           xv[u] = ld_keep_f32_if<true>(x + c[u], h, keep) + ld_keep_f32_if<false>(x + c[u], !h, keep);
         else  // joined as bits: a binary64 addition takes as long as the entry's own
-              // fma (R-MAT 2^22, 128 M entries: 541 us with it, 436 so)
+              // fma (R-MAT 2^22, 128 M entries: 541 us with it, 436 so,
+              // eight entries in flight)
           xv[u] = __longlong_as_double(
               __double_as_longlong(ld_keep_f64_if<true>(x + c[u], h, keep)) |
               __double_as_longlong(ld_keep_f64_if<false>(x + c[u], !h, keep)));
@@ -299,7 +307,7 @@ __device__ __forceinline__ void spmv_slice(const SpmvArgs& a, const int slice, c
 }
 
 template <int P, int VK, bool F64OUT>
-__global__ void __launch_bounds__(32 * SPMV_WPB) spmv_kernel(SpmvArgs a) {
+__global__ void __launch_bounds__(32 * SPMV_WPB, spmv_ctas_per_sm(P)) spmv_kernel(SpmvArgs a) {
   const int slice = blockIdx.x * SPMV_WPB + (threadIdx.x >> 5);
   if (slice >= a.nslices) return;
   spmv_slice<P, VK, F64OUT>(a, slice, threadIdx.x & 31);
