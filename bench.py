@@ -193,26 +193,26 @@ def make_inputs(args):
 
 # DRAM bytes per SpMV step (slice kernel + cut-row finaliser) measured by ncu
 # on the small case of the same kernels and layout (R-MAT scale 22, edge
-# factor 8, rows by degree: 557.4 MB against 605.8 MB of algorithmic bytes,
-# 0.920x; profiles/spmv_dram_fdf_rmat22_ef8.md) and scaled to this workload
+# factor 8, rows by degree: 558.2 MB against 605.8 MB of algorithmic bytes,
+# 0.921x; profiles/spmv_dram_fdf_rmat22_ef8.md) and scaled to this workload
 # by its algorithmic bytes per step (2,442,972,024: x 4.03); valid for the
 # kernel and layout sources whose SHA-256 is recorded with it
 SPMV_TRAFFIC = {
     "workload": "rmat24_ef8_normadj_seed1",
     "order": "degree",
-    "bytes_per_step": 2.248e9,
-    "measured_on": "rmat22_ef8_normadj_seed1 (557.4 MB per step), scaled by algorithmic bytes",
+    "bytes_per_step": 2.251e9,
+    "measured_on": "rmat22_ef8_normadj_seed1 (558.2 MB per step), scaled by algorithmic bytes",
     "sources": {
         "paper_2201_07498_gb300/csrc/te_spmv.cu":
-            "0ddeb9b3a8d19cd98cc189d7eb2a82f624f922edd1a0ad9b13b9a3ea11ef81ea",
+            "d4ac71a79b0e75ee2a4748070e5dff7aa7bf2946cb82be02f32e9d41f1b1c133",
         "paper_2201_07498_gb300/csrc/te_common.cuh":
-            "4a92b110c7810ee9286055e9629f3bb8af147b489cdb6326cff63482fe82bba1",
+            "765d884b2f7dea4a8aeedf6b5acf3147a7a148ff1a873a8e8af47ab3c151d034",
         "paper_2201_07498_gb300/csrc/te_layout.cu":
             "2e04e36f6ff8dddb6c1ec280a506a01b4a00e23d1e40214dc16daa4f7279106c",
         "paper_2201_07498_gb300/csrc/te_layout_dev.cu":
-            "b9794931a840a978b7559adc0fdccd1090315f9189c296e3e5a4ca4dde7a83e2",
+            "65ce101236588d1a6eb5839f7f8f981e29b18e84aa12ea62fd3e976d1291a4ea",
         "paper_2201_07498_gb300/csrc/te_internal.h":
-            "ee27e2ed3bc30a8907acafd806e9458318e59c3f91e7fbdc16be11a9f6e74a8c",
+            "7700d169f7ee75350f529359c011f98b676c4586f6609dde9375bd8c68bc0ae6",
     },
 }
 
