@@ -49,6 +49,7 @@ struct LzState {
   double c1[MAX_M + 2];     // coefficients of the first axpy pass
   double c2[MAX_M + 2];     // coefficients of the second axpy pass
   double xscale;            // multiplier of the source vector in the first axpy
+  double wnorm;             // binary64 form: the vector's norm after its first sweep
   double f2;                // delayed reorthogonalisation: coefficient of the candidate
   double bt[MAX_M + 2];     // delayed: norm of each candidate after one sweep
   int rflag[MAX_M + 2];     // delayed: column set by a restart (its beta is 0)

@@ -221,17 +221,26 @@ TE_DEV double acc_to_double(typename PassTr<P>::acc_t a) {
 // taken in binary32 (error 2^-24 2^LOW_BITS = 2^-60 of that scale, under the
 // binary64 rounding of the exact terms), off the binary64 pipe that would
 // bind the pass; otherwise in binary64 as before.  The scale: the largest
-// term of the update itself (the alpha and beta terms), |alpha| + beta for
-// the second sweep of a stored vector, the candidate for its own correction.
+// term of the update itself (the alpha and beta terms) for a first sweep; for
+// a second sweep the vector's own norm (of w after its first sweep, summed by
+// the pass that forms w; of the delayed form's candidate): what that sweep leaves
+// along the basis counts against the vector, which is far below |alpha| + beta
+// on a matrix close to a multiple of the identity.
 // Elements are scaled by their column's bound, so that binary32 holds them
 // whatever the matrix's magnitude; exponents outside what that covers, zero
 // scales and NaN take the binary64 form.  One warp per CTA, integers only.
 // R-MAT 2^22, 16 columns on average: the delayed form's update 284 -> 125 us
 // (5.25 TB/s; the binary64 pipe was 83 % busy at 27 % of the DRAM peak), the
 // solve 40.5 -> 34.9 ms; the Lanczos phase of 2^19 rows and 40 steps with both
-// sweeps 9.58 -> 8.52 ms.  Error against 64 bits unchanged (4.3e-14 and 5.0e-14
+// sweeps 9.58 -> 8.46 ms.  Error against 64 bits unchanged (4.3e-14 and 5.0e-14
 // for the former's vectors, 1.2e-15 for the latter's basis).
+// From four columns and two tiles per CTA on: the search and the norm's sum
+// cost a CTA about 1 us per step, what they save comes with every tile.  Solves with
+// both sweeps, m 40, in binary64 alone and by this rule: 524,287 rows (13 tiles)
+// 7.52 and 6.51 ms, 100,000 (2.6) 3.20 and 3.03, 60,000 (1.5) 2.82 and 2.74; 10,000
+// rows, a tile per CTA, m 16: 0.77 ms against 0.80 with binary32 there too.
 constexpr int LOW_BITS = -36;
+constexpr int LOW_COLS = 4, LOW_TILES = 1;  // at least, and more than
 
 TE_DEV int biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 // a bound on the (biased) exponents of a column with scale s = 1 / norm
@@ -270,8 +279,7 @@ TE_DEV void low_coefs(const PassArgs& a, LowCoef* lc, int* info, int lane) {
     ref = st->f2 != 0.0 ? biased_exp(st->f2) + ec : 0;
     emin = emax = ec;
   }
-  if (MODE == MODE_AXPY_STORE)
-    ref = biased_exp(fabs(st->alpha[a.step]) + st->beta[a.step]) + 1023;
+  if (MODE == MODE_AXPY_STORE) ref = biased_exp(st->wnorm) + 1023;
   bool fine = true;
   for (int j = lane; j < ncol; j += 32) {
     const int ec = column_exp(st->s[a.col0 + j]);
@@ -822,8 +830,13 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
   }
   LowCoef* lowc = reinterpret_cast<LowCoef*>(sm + L.low_off);
   int* lowinfo = abortflag + 1;  // whether the small coefficients go in binary32; two exponents
+  const bool lowpass = P == PREC_DDD && nb >= LOW_COLS && tiles > (int64_t)LOW_TILES * ncta;
   if constexpr (P == PREC_DDD && (HAS_AXPY || DUPD)) {
-    if (wid == 0) low_coefs<MODE>(a, lowc, lowinfo, lane);
+    if (!lowpass) {
+      if (tid == 0) lowinfo[0] = 0;
+    } else if (wid == 0) {
+      low_coefs<MODE>(a, lowc, lowinfo, lane);
+    }
   }
   // Ritz coefficients C (nb x K) with the row stride padded to Kp (a multiple
   // of RITZ_KC, zeros beyond K); FDF keeps their binary32 roundings only
@@ -1048,6 +1061,8 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
             // the second-sweep dot of column i (it enters alpha_i) is exact; a
             // thread per row keeps the warps of phase B balanced
             dacc_fma(n1, tv[(size_t)(nb - 1) * TILE_R + tid], w.x, w.y);
+          } else {
+            n1 = fma(w, w, n1);  // ||w||^2, the second sweep's scale
           }
         } else {
           // store the next basis vector (unnormalised) and its two norms
@@ -1411,14 +1426,16 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
       }
     }
   }
-  if constexpr (MODE == MODE_AXPY_DOT && P == PREC_FDF) {
+  // the second sweep's scale, where that sweep may use it
+  const bool wnorm = MODE == MODE_AXPY_DOT && lowpass;
+  if (MODE == MODE_AXPY_DOT && (P == PREC_FDF || wnorm)) {
     n1 = warp_sum(n1);
     if (lane == 0) red[wid] = n1;
     named_bar_sync(1, CONSUMERS);
     if (tid == 0) {
       acc_t t1 = red[0];
       for (int w = 1; w < CONSUMERS / 32; ++w) t1 = acc_merge<P>(t1, red[w]);
-      put_partial<P>(a.partials, pidx(nb - 1, cta, ncta), t1);
+      put_partial<P>(a.partials, pidx(P == PREC_FDF ? nb - 1 : SLOT_N, cta, ncta), t1);
     }
   }
   if constexpr (MODE == MODE_AXPY_STORE || DUPD || DDOT) {
@@ -1456,10 +1473,11 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
   named_bar_sync(1, CONSUMERS);
   if (*lastflag == 0) return;
   __threadfence();
-  const int slots = (MODE == MODE_AXPY_STORE || DUPD) ? 2 : (DDOT ? 2 * nb : nb);
+  const int slots = (MODE == MODE_AXPY_STORE || DUPD) ? 2 : (DDOT ? 2 * nb : nb + (wnorm ? 1 : 0));
   for (int q = wid; q < slots; q += CONSUMERS / 32) {
     const int slot = (MODE == MODE_AXPY_STORE || DUPD) ? SLOT_N + q
                      : (DDOT && q >= nb)               ? SLOT_D2 + (q - nb)
+                     : (wnorm && q == nb)              ? SLOT_N
                                                        : q;
     acc_t acc = zero_acc<P>();
     // each lane adds the CTAs lane, lane + 32, ... in order; a chunk's loads
@@ -1479,6 +1497,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
     if (lane == 0) tot[q] = acc_to_double<P>(acc);
   }
   named_bar_sync(1, CONSUMERS);
+  if (wnorm && tid == 0) st->wnorm = sqrt(tot[nb]);
   finalize_pass(a, tot, reinterpret_cast<double*>(sm + L.fin_off), tid);
   if (tid == 0) {
     st->ticket = 0;
