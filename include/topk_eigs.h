@@ -61,7 +61,12 @@ typedef enum {
 typedef enum { TE_F64 = 0, TE_F32 = 1, TE_BF16 = 2, TE_FP8_E4M3 = 3 } te_dtype;
 
 /* (matrix values, arithmetic, vector storage).  Supported:
- *   DDD = {TE_F64, TE_F64, TE_F64}: plain binary64 on the FP64 pipe.
+ *   DDD = {TE_F64, TE_F64, TE_F64}: binary64 data, vectors and results.  The
+ *         basis passes replace binary64 arithmetic where the error stays below
+ *         its rounding: update terms below 2^-45 of the update's scale are
+ *         taken in binary32, dots and Ritz sums over enough columns in 61-bit
+ *         fixed point relative to the largest element of a vector, column or
+ *         row (an element far below that keeps fewer bits of its own).
  *   FDD = {TE_F32, TE_F64, TE_F64}: as DDD with binary32 matrix values
  *         (converted exactly to binary64 as they are read).
  *   FDF = {TE_F32, TE_F64, TE_F32}: binary32 matrix values and Lanczos

@@ -23,8 +23,8 @@
 // reduces them in a fixed order and computes the next pass's coefficients,
 // alpha, beta and the breakdown flag on the device - no host round trip.
 //
-// Precision: DDD uses binary64 FMA (and binary32 for updates whose terms all
-// lie below 2^-36 of the result, see low_coefs).  FDF stores V in binary32 and carries
+// Precision: DDD uses binary64 FMA (and binary32 for an update's small terms where
+// all of them lie below 2^-45 of its scale, see low_coefs).  FDF stores V in binary32 and carries
 // every product and sum in double-float (te_common.cuh); per-CTA partials are
 // double-float, the final cross-CTA sums binary64.
 #include "te_common.cuh"
@@ -218,9 +218,13 @@ TE_DEV double acc_to_double(typename PassTr<P>::acc_t a) {
 // orthogonal, all but the last two coefficients sit at the rounding level (of
 // the order of 1e-15), and their products need only a few digits: where every
 // one of them is below 2^LOW_BITS of the update's scale, the products are
-// taken in binary32 (error 2^-24 2^LOW_BITS = 2^-60 of that scale, under the
-// binary64 rounding of the exact terms), off the binary64 pipe that would
-// bind the pass; otherwise in binary64 as before.  The scale: the largest
+// taken in binary32, off the binary64 pipe that would bind the pass; with one
+// that is not, all are taken in binary64.  The rule compares exponents, so that
+// a coefficient times its column's norm may reach 2^(LOW_BITS + 2) of the scale;
+// its two factors are cut to 24 bits (2^-22 together) and a chain's up to 18
+// sums rounded (2^-19.8), so 62 such columns are off by at most 2^(LOW_BITS + 8
+// - 19.6) = 2^-56.6 of the scale, a tenth of the binary64 rounding of the exact
+// terms beside them.  The scale: the largest
 // term of the update itself (the alpha and beta terms) for a first sweep; for
 // a second sweep the vector's own norm (of w after its first sweep, summed by
 // the pass that forms w; of the delayed form's candidate): what that sweep leaves
@@ -239,7 +243,7 @@ TE_DEV double acc_to_double(typename PassTr<P>::acc_t a) {
 // both sweeps, m 40, in binary64 alone and by this rule: 524,287 rows (13 tiles)
 // 7.52 and 6.51 ms, 100,000 (2.6) 3.20 and 3.03, 60,000 (1.5) 2.82 and 2.74; 10,000
 // rows, a tile per CTA, m 16: 0.77 ms against 0.80 with binary32 there too.
-constexpr int LOW_BITS = -36;
+constexpr int LOW_BITS = -45;
 constexpr int LOW_COLS = 4, LOW_TILES = 1;  // at least, and more than
 
 TE_DEV int biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
@@ -312,7 +316,7 @@ TE_DEV void low_coefs(const PassArgs& a, LowCoef* lc, int* info, int lane) {
   for (int j = lane; j < ncol; j += 32) {
     const int ec = column_exp(st->s[a.col0 + j]);
     LowCoef o;
-    // c 2^(ec - 1023 - r): at most 2^LOW_BITS where it is used
+    // c 2^(ec - 1023 - r): at most 2^(LOW_BITS + 1) where it is used
     o.c2 = j < nsmall && c2[j] != 0.0 ? low_word(c2[j], (896 + r - (ec - 1023)) * (1 << 20)) : 0.f;
     o.c1 = DUPD && c1[j] != 0.0 ? low_word(c1[j], (896 + r1 - (ec - 1023)) * (1 << 20)) : 0.f;
     o.bias = (ec - 127) * (1 << 20);  // an element times 2^-(ec - 1023), below 1 in magnitude
