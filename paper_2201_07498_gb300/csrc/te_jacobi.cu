@@ -454,8 +454,17 @@ __global__ void __launch_bounds__(JAC_THREADS, 1) jacobi_kernel(JacobiArgs a) {
     cluster_barrier();
     if (rank != 0) return;
   }
-  const double* const theta = sm.diag[buf];
+  // The Ritz values, unscaled.  Divided by 2^texp, a diagonal element below 2^-1022
+  // of the largest has lost bits; a rotation would have moved it by at least
+  // 1e-33 of ||T||, so that one still there (or lost entirely) is alpha itself.
+  double* const theta = sm.diag[buf ^ 1];
   int* const sel = sm.sel;
+  constexpr int64_t NORMAL = (int64_t)1 << 52;
+  if (tid < m) {
+    const double d = sm.diag[buf][tid];
+    const bool lost = abs_bits(d) < NORMAL && abs_bits(t_init(tid, tid)) < NORMAL;
+    theta[tid] = lost ? a.alpha[tid] : scalbn(d, texp);
+  }
 
   // selection: rank of each Ritz value under the selection order
   if (tid < m) sm.key[tid] = order_key(theta[tid]);
@@ -494,7 +503,7 @@ __global__ void __launch_bounds__(JAC_THREADS, 1) jacobi_kernel(JacobiArgs a) {
     }
     const int64_t flip = __double_as_longlong(Y[bi * JLD + j]) & INT64_MIN;
     if (lane == 0) {
-      const double th = scalbn(theta[j], texp);
+      const double th = theta[j];
       a.theta_out[k] = th;
       if (eigvals_dev) eigvals_dev[k] = th;
       if (a.resid_out) a.resid_out[k] = fabs(a.beta[m] * Y[(m - 1) * JLD + j]);
