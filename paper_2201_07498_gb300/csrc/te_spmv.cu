@@ -186,14 +186,24 @@ constexpr int SPMV_WPB = 8;     // warps (slices) per CTA
 // with rows relabelled by degree, the first HOT_BYTES of x (the most
 // connected columns) are the ones L1 keeps
 constexpr int64_t HOT_BYTES = 128 << 10;
-// Entries per lane in flight, and the CTAs per SM that the registers are held to:
-// the gathers' latency is hidden better by more warps than by more loads per warp
-// (unless registers spill).  R-MAT 2^22, 128 M entries, rows by degree, us per SpMV
-// with 8 entries and free registers / 4 and free / 4 and 6 CTAs / 4 and 8 CTAs: DDD
-// 431 / 395 / 375 / 415, FDF 291 / 296 / 295 / 286, 8DF 313 / 296 / 296 / 282.  The
-// order of a row's sum does not depend on it (entries alternate between two chains).
-constexpr int SPMV_UNROLL = 4;
-constexpr int spmv_ctas_per_sm(int prec) { return prec == PREC_DDD ? 6 : 8; }
+// Two forms of the kernel: WIDE has eight entries per lane in flight and free
+// registers, MANY four entries and registers held to six or eight CTAs per SM.
+// The order of a row's sum is the same (entries alternate between two chains).
+// With the gathers split into hot and cold columns (rows by degree) MANY hides
+// their latency better once its warps are all at work: R-MAT 2^22, 128 M entries,
+// us per SpMV, WIDE / MANY: DDD 431 / 375, FDF 291 / 286, 8DF 313 / 282.  In the
+// caller's order, and with too few slices for the warps to fill, a slice's own
+// chain of chunks sets the end: WIDE / MANY, caller's order, R-MAT, 32 entries per
+// row, 50,000 rows FDF 18.8 / 25.0, DDD 21.0 / 24.9, 300,000 rows DDD 44.8 / 55.8,
+// BDF 42.2 / 46.3, 1.5 M rows within 4 %; by degree, R-MAT and uniform rows, slices per
+// SM: DDD 41-62 0.91-1.08 times WIDE's speed, 80-113 1.09-1.14, 156-308 1.04-1.16; binary32
+// arithmetic 40-62 0.93-1.08, 80-113 0.92-1.00, 156-164 1.00-1.12, 283-308 1.01-1.16.
+constexpr int SPMV_WIDE = 8, SPMV_MANY = 4;
+constexpr int spmv_ctas_per_sm(int prec, int unroll) {
+  return unroll == SPMV_WIDE ? 1 : prec == PREC_DDD ? 6 : 8;
+}
+// MANY from this many slices per SM on, rows by degree
+constexpr int spmv_many_slices(int prec) { return prec == PREC_DDD ? 72 : 128; }
 
 // stored matrix value type per te_dtype, and its streaming load + exact
 // conversion to the arithmetic's input type
@@ -228,7 +238,7 @@ TE_DEV auto load_value(const typename VStore<VK>::t* p, uint64_t pol) {
 // rows are summed over their codes and multiplied by the row scale at the end.
 // one warp sums one slice (lane = one piece); the serving engine's batched
 // SpMV runs the same body on the slices of several solves
-template <int P, int VK, bool F64OUT>
+template <int P, int VK, bool F64OUT, int UNROLL>
 __device__ __forceinline__ void spmv_slice(const SpmvArgs& a, const int slice, const int lane) {
   using Tr = SpmvTr<P>;
   using val_t = typename Tr::val_t;
@@ -254,20 +264,20 @@ __device__ __forceinline__ void spmv_slice(const SpmvArgs& a, const int slice, c
       acc = fma(v, xv, acc);
     }
   };
-  // chunks of SPMV_UNROLL entries per lane; all loads of a chunk go out
+  // chunks of UNROLL entries per lane; all loads of a chunk go out
   // before its gathers, and the tail of a slice is a predicated chunk
-  for (int k = 0; k < sl.len; k += SPMV_UNROLL) {
-    int32_t c[SPMV_UNROLL];
-    val_t v[SPMV_UNROLL];
+  for (int k = 0; k < sl.len; k += UNROLL) {
+    int32_t c[UNROLL];
+    val_t v[UNROLL];
 #pragma unroll
-    for (int u = 0; u < SPMV_UNROLL; ++u) {
+    for (int u = 0; u < UNROLL; ++u) {
       const bool ok = k + u < sl.len;
       c[u] = ok ? ld_stream_i32(cp + (int64_t)(k + u) * SELL_C, pol) : 0;
       v[u] = ok ? (val_t)load_value<VK>(vp + (int64_t)(k + u) * SELL_C, pol) : (val_t)0;
     }
-    x_t xv[SPMV_UNROLL];
+    x_t xv[UNROLL];
 #pragma unroll
-    for (int u = 0; u < SPMV_UNROLL; ++u) {  // padding reads x[0]
+    for (int u = 0; u < UNROLL; ++u) {  // padding reads x[0]
       if (a.hot > 0) {  // uniform: cold columns leave L1 to the hot ones
         const bool h = c[u] < a.hot;
         if constexpr (sizeof(x_t) == 4)
@@ -284,7 +294,7 @@ __device__ __forceinline__ void spmv_slice(const SpmvArgs& a, const int slice, c
       }
     }
 #pragma unroll
-    for (int u = 0; u < SPMV_UNROLL; u += 2) {
+    for (int u = 0; u < UNROLL; u += 2) {
       add(acc0, v[u], xv[u]);
       add(acc1, v[u + 1], xv[u + 1]);
     }
@@ -306,11 +316,12 @@ __device__ __forceinline__ void spmv_slice(const SpmvArgs& a, const int slice, c
   }
 }
 
-template <int P, int VK, bool F64OUT>
-__global__ void __launch_bounds__(32 * SPMV_WPB, spmv_ctas_per_sm(P)) spmv_kernel(SpmvArgs a) {
+template <int P, int VK, bool F64OUT, int UNROLL>
+__global__ void __launch_bounds__(32 * SPMV_WPB, spmv_ctas_per_sm(P, UNROLL))
+    spmv_kernel(SpmvArgs a) {
   const int slice = blockIdx.x * SPMV_WPB + (threadIdx.x >> 5);
   if (slice >= a.nslices) return;
-  spmv_slice<P, VK, F64OUT>(a, slice, threadIdx.x & 31);
+  spmv_slice<P, VK, F64OUT, UNROLL>(a, slice, threadIdx.x & 31);
 }
 
 // Cut rows: the first nbig rows (most pieces first) get a whole warp each:
@@ -385,8 +396,15 @@ __global__ void spmv_long_finalize(const LongRow* lrows, int nl, int nbig, int b
 
 template <int P, int VK, bool F64OUT>
 static cudaError_t launch_spmv_t(const SpmvArgs& a, const DevSell& S, cudaStream_t s) {
-  if (S.nslices > 0)
-    spmv_kernel<P, VK, F64OUT><<<(S.nslices + SPMV_WPB - 1) / SPMV_WPB, 32 * SPMV_WPB, 0, s>>>(a);
+  if (S.nslices > 0) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const bool many = a.hot > 0 && S.nslices / sms >= spmv_many_slices(P);
+    auto* k = many ? spmv_kernel<P, VK, F64OUT, SPMV_MANY> : spmv_kernel<P, VK, F64OUT, SPMV_WIDE>;
+    k<<<(S.nslices + SPMV_WPB - 1) / SPMV_WPB, 32 * SPMV_WPB, 0, s>>>(a);
+  }
   if (S.nlrows > 0) {
     const int threads = 256;
     const int big_blocks = (int)(((int64_t)S.nlbig * 32 + threads - 1) / threads);
@@ -456,8 +474,8 @@ __global__ void __launch_bounds__(32 * SPMV_WPB) batch_spmv_kernel(const BatchTa
     a.nslices = B.nslices;
     a.hot = 0;
     const int slice = (int)(g - c.off[sidx]);
-    if (B.vk == TE_BF16) spmv_slice<PREC_FDF, TE_BF16, false>(a, slice, lane);
-    else spmv_slice<PREC_FDF, TE_F32, false>(a, slice, lane);
+    if (B.vk == TE_BF16) spmv_slice<PREC_FDF, TE_BF16, false, SPMV_WIDE>(a, slice, lane);
+    else spmv_slice<PREC_FDF, TE_F32, false, SPMV_WIDE>(a, slice, lane);
   }
 }
 
