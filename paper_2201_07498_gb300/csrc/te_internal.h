@@ -306,6 +306,7 @@ struct PassLaunch {
   size_t smem = 0;
   size_t region = 0;  // bytes of the stage buffers
   int stages = 0;
+  size_t dig_smem = 0, dig_region = 0;  // the same with DDD dots in digits
 };
 // configure a pass kernel for `max_cols` basis columns (and K Ritz vectors);
 // returns the launch shape

@@ -123,7 +123,8 @@ struct SmemPlan {
 // finalize scratch (doubles): copies of s, alpha, beta, the c_j, warp sums
 constexpr int FIN_SCRATCH = 4 * (MAX_M + 2) + 2 * (CONSUMERS / 32) + 8;
 // ritz_elems: m*K coefficients held by the Ritz pass (0 for the other passes)
-__host__ __device__ inline SmemPlan smem_plan(int prec, int mode, size_t region, int ritz_elems) {
+__host__ __device__ inline SmemPlan smem_plan(int mode, bool digits, size_t region,
+                                              int ritz_elems) {
   SmemPlan p{};
   p.region = region;
   p.ws_off = align_up(region, 128);
@@ -132,11 +133,11 @@ __host__ __device__ inline SmemPlan smem_plan(int prec, int mode, size_t region,
   p.ritz_off = p.coef2_off + (MAX_M + 2) * 8;
   size_t ritz = (mode == MODE_RITZ) ? align_up((size_t)ritz_elems * 8, 128) : 0;
   p.red_off = p.ritz_off + ritz;
-  p.fin_off = align_up(p.red_off + PSTRIDE * 8, 8);
-  const bool ddd = prec == PREC_DDD && mode != MODE_RITZ;
+  // (the tiles' small coefficients and the epilogue's scratch share their room)
+  static_assert(sizeof(LowCoef) * MAX_M <= FIN_SCRATCH * 8, "");
+  p.low_off = p.fin_off = align_up(p.red_off + PSTRIDE * 8, alignof(LowCoef));
   p.dig_off = align_up(p.fin_off + FIN_SCRATCH * 8, alignof(DigitBuf));
-  p.low_off = align_up(p.dig_off + (has_digits(prec, mode) ? sizeof(DigitBuf) : 0), alignof(LowCoef));
-  p.bar_off = align_up(p.low_off + (ddd ? sizeof(LowCoef) * MAX_M : 0), 8);
+  p.bar_off = align_up(p.dig_off + (digits ? sizeof(DigitBuf) : 0), 8);
   p.total = p.bar_off + 2 * MAX_STAGES * 8 + 32;
   return p;
 }
@@ -364,6 +365,9 @@ constexpr int INT_ROWS = 256;
 // over 0 ... 31 columns, binary64 dots and digits: 2^22 rows 9.64 and 7.26 ms, 2^20
 // (27 tiles per CTA) 2.99 and 2.49, 2^18 (6.7) 1.35 and 1.30; 150,001 rows (3.9)
 // 1.12 and about 1.15.  From 7, 9 or 13 columns on, 2^20 rows: 2.49, 2.50, 2.52.
+// More columns, us per pass over 40-44, 49-53 and 59-63 of them: 2^18 rows 80, 90 and
+// 117 in binary64, 69, 82 and 84 in digits; 2^20 201, 237 and 310, 159, 205 and 210;
+// 2^22 682, 806 and 1,084, 510, 662 and 693 (one stage from 46 columns on).
 constexpr int IDOT_TILES = 6, IDOT_COLS = 8;
 
 // the bound on the exponents of a column with scale s (1 / norm): |x| <= norm,
@@ -752,7 +756,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, size_t region, cons
     if (*((volatile int*)&st->restart_flag) == 0) return;
   }
   const SmemPlan L = smem_plan(
-      P, MODE, region, MODE == MODE_RITZ ? a.nb * ((a.K + RITZ_KC - 1) / RITZ_KC * RITZ_KC) : 0);
+      MODE, DIG, region, MODE == MODE_RITZ ? a.nb * ((a.K + RITZ_KC - 1) / RITZ_KC * RITZ_KC) : 0);
   vec_t* ws = reinterpret_cast<vec_t*>(sm + L.ws_off);
   coef_t* coef = reinterpret_cast<coef_t*>(sm + L.coef_off);
   coef_t* coef2 = reinterpret_cast<coef_t*>(sm + L.coef2_off);
@@ -1823,28 +1827,35 @@ static cudaError_t config_t(int max_cols, int K, int num_sms, PassLaunch& out) {
   const int ritz_elems = MODE == MODE_RITZ ? max_cols * ((K + RITZ_KC - 1) / RITZ_KC * RITZ_KC) : 0;
   // pass_ctas_per_sm CTAs per SM share the SM's shared memory (minus the
   // per-CTA reservation of 1 KB)
-  const size_t fixed = smem_plan(P, MODE, 0, ritz_elems).total + 128;
   int persm = 0;
   e = cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e != cudaSuccess) return e;
   const size_t half = (size_t)persm / pass_ctas_per_sm(P) - 1024;
   const size_t cap = half < (size_t)optin ? half : (size_t)optin;
-  size_t avail = cap > fixed ? cap - fixed : 0;
   // a stage: max_cols basis columns of a tile, plus the pass vector's rows
   const size_t per_stage = (size_t)(max_cols > 0 ? max_cols : 1) * TILE_R * sizeof(basis_t) +
                            (MODE == MODE_RITZ ? 0 : (size_t)TILE_R * 8);
   // every byte that fits: the kernel fits region / (its stage) stages, so
   // that passes over few columns keep many tiles in flight
-  const size_t region = avail / 128 * 128;
-  const int stages = (int)(region / per_stage);
+  auto plan = [&](bool digits, size_t& region, size_t& total) {
+    const size_t fixed = smem_plan(MODE, digits, 0, ritz_elems).total + 128;
+    region = (cap > fixed ? cap - fixed : 0) / 128 * 128;
+    total = smem_plan(MODE, digits, region, ritz_elems).total;
+    return (int)(region / per_stage);
+  };
+  size_t region = 0, total = 0;
+  const int stages = plan(false, region, total);
   if (stages < 1) return cudaErrorInvalidConfiguration;
-  const size_t total = smem_plan(P, MODE, region, ritz_elems).total;
   e = cudaFuncSetAttribute(pass_kernel<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)total);
   if (e != cudaSuccess) return e;
   if constexpr (has_digits(P, MODE)) {
+    // the digits' buffers cost a stage from 46 columns on (the binary64 form has
+    // two up to 54: 200,000 rows, 54 steps, 2.90 ms of dot passes with their room
+    // reserved there too, 2.85 without)
+    if (plan(true, out.dig_region, out.dig_smem) < 1) return cudaErrorInvalidConfiguration;
     e = cudaFuncSetAttribute(pass_kernel<P, MODE, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)total);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out.dig_smem);
     if (e != cudaSuccess) return e;
   }
   if constexpr (P == PREC_DDD && MODE == MODE_RITZ) {
@@ -1893,7 +1904,7 @@ cudaError_t launch_pass(int prec, int mode, const PassArgs& a, const PassLaunch&
       dig = a.nb - 1 >= IDOT_COLS && a.ld / TILE_R >= (int64_t)IDOT_TILES * L.grid; \
     if (dig)                                                                     \
       pass_kernel<PP, MM, has_digits(PP, MM)>                                    \
-          <<<L.grid, PASS_THREADS, L.smem, s>>>(a, L.region);                    \
+          <<<L.grid, PASS_THREADS, L.dig_smem, s>>>(a, L.dig_region);            \
     else                                                                         \
       pass_kernel<PP, MM><<<L.grid, PASS_THREADS, L.smem, s>>>(a, L.region);     \
     return cudaGetLastError();                                                   \
