@@ -604,7 +604,10 @@ extern "C" te_status te_spmv_noalloc(const te_csr* A, te_precision p, const void
   status[1] = 0;
   e = prec == PREC_DDD ? na_launch<PREC_DDD>(A, x, y, nchunks, scratch, status_dev, s)
                        : na_launch<PREC_FDF>(A, x, y, nchunks, scratch, status_dev, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  // also after a launch that failed: a kernel queued before it may still set the
+  // slot's words, which the next call to take the slot would read
+  const cudaError_t es = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return fail(TE_ERR_CUDA, std::string("te_spmv_noalloc: ") + cudaGetErrorString(e));
   if (status[1]) return fail(TE_ERR_INVALID_ARG, "te_spmv_noalloc: malformed row_ptr");
   if (status[0]) return fail(TE_ERR_INVALID_ARG, "te_spmv_noalloc: a column index is outside [0, n)");
