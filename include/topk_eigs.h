@@ -312,10 +312,14 @@ te_status te_tridiag_eigs(int32_t m, const double* alpha, const double* beta, in
  * for such callers.  Work memory is one fixed 4 MiB __device__ array inside
  * the library, shared by all calls on a device, which limits nnz to
  * 131072 * 2048 (DDD) or 131072 * 4096 (FDF); larger matrices get
- * TE_ERR_INVALID_ARG.  The first call on each device looks up the array's
- * device address (do that first call before any stream capture); the
- * address is kept for the life of the process, so a program that resets a
- * device (cudaDeviceReset) must not call this entry point on it afterwards.
+ * TE_ERR_INVALID_ARG.  A call's status words lie in a fixed managed array of
+ * 32 KB, loaded with the library.  The first call on each device looks up the
+ * work memory's device address and allows the kernels their shared memory (do
+ * that first call before any stream capture); the address is kept for the
+ * life of the process, so a program that resets a device (cudaDeviceReset)
+ * must not call this entry point on it afterwards.  Up to 64 calls per device
+ * may be inside this function at once (their work ordered on the GPU, see
+ * below); further ones wait for one of them to return.
  * Calls that overlap on the GPU (other streams, other host threads) race on
  * the array and must be serialised by the caller.  A must be TE_DEVICE with
  * values_f64 = 0 (there is no room to round the values); x has n elements of

@@ -332,6 +332,11 @@ struct JacobiArgs {
 cudaError_t jacobi_prepare();  // once per process/device, outside stream capture
 cudaError_t launch_jacobi(const JacobiArgs& a, cudaStream_t s);
 
+// ---- te_spmv_noalloc's status words (te_noalloc_status.cu) ----
+constexpr int NA_DEVICES = 64;  // devices
+constexpr int NA_SLOTS = 64;    // calls in flight per device (further ones wait)
+int* noalloc_status_words();    // two per slot, [device][slot][2]
+
 // ---- Rayleigh-quotient refinement and Gram matrix ----
 // The K Ritz vectors U (binary64, by rows, row stride K rounded up to even)
 // against the binary64 matrix S: replaces st->theta_sel[k] by the Rayleigh

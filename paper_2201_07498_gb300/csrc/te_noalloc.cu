@@ -452,7 +452,7 @@ constexpr int64_t NA_SEARCH_CHUNKS = 2048;
 // that need no opt-in) is allowed on this device by na_prepare
 template <int P>
 static cudaError_t na_launch(const te_csr* A, const void* x, double* y, int64_t nchunks,
-                             unsigned char* scratch, int* status_dev, cudaStream_t s) {
+                             unsigned char* scratch, int* status, cudaStream_t s) {
   constexpr int CH = NaTr<P>::CHUNK;
   const int chunk_blocks = (int)((nchunks + 7) / 8);
   if (nchunks > 0) {
@@ -464,13 +464,13 @@ static cudaError_t na_launch(const te_csr* A, const void* x, double* y, int64_t 
                        reinterpret_cast<uintptr_t>(A->values)) & 15) == 0;
     auto* k = vec ? noalloc_chunk_kernel<P, true> : noalloc_chunk_kernel<P, false>;
     k<<<(unsigned)nchunks, NOALLOC_THREADS, sizeof(NaSmem<P>), s>>>(
-        A->row_ptr, A->col_idx, A->values, x, y, A->n, A->nnz, searched, scratch, status_dev);
+        A->row_ptr, A->col_idx, A->values, x, y, A->n, A->nnz, searched, scratch, status);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   const int64_t row_blocks = (A->n + 256 * NA_FIX_ROWS - 1) / (256 * NA_FIX_ROWS);
   noalloc_fixup_kernel<P><<<(unsigned)(chunk_blocks + row_blocks), 256, 0, s>>>(
-      A->row_ptr, y, A->n, A->nnz, nchunks, chunk_blocks, scratch, status_dev);
+      A->row_ptr, y, A->n, A->nnz, nchunks, chunk_blocks, scratch, status);
   return cudaGetLastError();
 }
 
@@ -486,20 +486,16 @@ static cudaError_t na_prepare() {
 }
 
 namespace {
-// Per device: the scratch array's address and the status words (bad column,
-// malformed row_ptr) in pinned host memory that the kernels write straight
-// into, only when something is wrong.  The host clears a call's words before
-// it and reads them after its synchronisation, so a call is two launches and
-// a wait: a status word on the device took a memset and a copy more (53 us
-// against 32 us a call at 600 k entries).  Every call in flight has a slot of
-// its own.
-constexpr int NA_SLOTS = 64;      // calls in flight per device (further ones wait)
-constexpr int NA_SLOT_INTS = 16;  // a slot: 64 bytes
+// Per device: the scratch array's address and the calls in flight.  A call's
+// status words (bad column, malformed row_ptr) lie in managed memory, which the
+// kernels write straight into, only when something is wrong.  The host clears
+// them before the call and reads them after its synchronisation, so a call is
+// two launches and a wait: a status word on the device took a memset and a copy
+// more (53 us against 32 us a call at 600 k entries).  Every call in flight has
+// a slot of its own.
 struct NaDevice {
   void* scratch = nullptr;
-  int* status = nullptr;      // host address of slot 0
-  int* status_dev = nullptr;  // the same words as the device addresses them
-  uint64_t busy = 0;          // one bit per slot
+  uint64_t busy = 0;  // one bit per slot
 };
 std::mutex g_na_mu;
 std::condition_variable g_na_cv;
@@ -524,6 +520,7 @@ struct NaSlot {
   }
 };
 static_assert(NA_SLOTS == 64, "one bit of `busy` per slot");
+static_assert(NA_DEVICES >= NOALLOC_MAX_DEVICES, "status words for every device");
 }  // namespace
 
 }  // namespace te
@@ -569,12 +566,12 @@ extern "C" te_status te_spmv_noalloc(const te_csr* A, te_precision p, const void
   if (dev < 0 || dev >= NOALLOC_MAX_DEVICES)
     return fail(TE_ERR_UNSUPPORTED, "te_spmv_noalloc: device index too large");
   // once per device, with that device current: the scratch array's device
-  // address and the status words (kept for the life of the process; a device
-  // reset invalidates them)
+  // address (kept for the life of the process; a device reset invalidates it)
+  // and the chunk kernels' shared memory
   NaDevice& g = g_na[dev];
   {
     std::lock_guard<std::mutex> lk(g_na_mu);
-    if (!g.status) {
+    if (!g.scratch) {
       void* ptr = nullptr;
       e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
       if (e != cudaSuccess)
@@ -583,27 +580,17 @@ extern "C" te_status te_spmv_noalloc(const te_csr* A, te_precision p, const void
       if (e == cudaSuccess) e = na_prepare<PREC_FDF>();
       if (e != cudaSuccess)
         return fail(TE_ERR_CUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
-      int* st = nullptr;
-      void* st_dev = nullptr;
-      e = cudaHostAlloc(reinterpret_cast<void**>(&st), NA_SLOTS * NA_SLOT_INTS * sizeof(int),
-                        cudaHostAllocMapped);
-      if (e == cudaSuccess && (e = cudaHostGetDevicePointer(&st_dev, st, 0)) != cudaSuccess)
-        cudaFreeHost(st);
-      if (e != cudaSuccess)
-        return fail(TE_ERR_CUDA, std::string("status words: ") + cudaGetErrorString(e));
       g.scratch = ptr;
-      g.status = st;
-      g.status_dev = static_cast<int*>(st_dev);
     }
   }
   NaSlot slot(g);
   unsigned char* scratch = static_cast<unsigned char*>(g.scratch);
-  volatile int* status = g.status + slot.i * NA_SLOT_INTS;
-  int* status_dev = g.status_dev + slot.i * NA_SLOT_INTS;
+  int* words = noalloc_status_words() + (dev * NA_SLOTS + slot.i) * 2;
+  volatile int* status = words;
   status[0] = 0;
   status[1] = 0;
-  e = prec == PREC_DDD ? na_launch<PREC_DDD>(A, x, y, nchunks, scratch, status_dev, s)
-                       : na_launch<PREC_FDF>(A, x, y, nchunks, scratch, status_dev, s);
+  e = prec == PREC_DDD ? na_launch<PREC_DDD>(A, x, y, nchunks, scratch, words, s)
+                       : na_launch<PREC_FDF>(A, x, y, nchunks, scratch, words, s);
   // also after a launch that failed: a kernel queued before it may still set the
   // slot's words, which the next call to take the slot would read
   const cudaError_t es = cudaStreamSynchronize(s);

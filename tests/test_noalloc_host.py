@@ -37,6 +37,10 @@ static cudaError_t fake_host_alloc(void** p, size_t b) {
 #define cudaFreeHost(p) fake_ok()
 #include "te_noalloc.cu"
 void te::set_last_error(const std::string&) {}
+int* te::noalloc_status_words() {
+  static int words[NA_DEVICES * NA_SLOTS * 2];
+  return words;
+}
 
 int main(int argc, char** argv) {
   fail_launch = atoi(argv[1]);
@@ -83,3 +87,8 @@ def test_call_ends_after_what_it_queued(call, fail_launch):
     r = call(fail_launch)
     assert (r["rc"] == 0) == (fail_launch == 0)
     assert r["sync"] == 1
+
+
+def test_call_allocates_nothing(call):
+    # neither on the device nor page-locked on the host, not even the first time
+    assert call(0)["alloc"] == 0
