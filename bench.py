@@ -194,7 +194,7 @@ def make_inputs(args):
 # DRAM bytes per SpMV step (slice kernel + cut-row finaliser) measured by ncu
 # on the small case of the same kernels and layout (R-MAT scale 22, edge
 # factor 8, rows by degree: 558.2 MB against 605.8 MB of algorithmic bytes,
-# 0.921x; profiles/spmv_dram_fdf_rmat22_ef8.md) and scaled to this workload
+# 0.921x) and scaled to this workload
 # by its algorithmic bytes per step (2,442,972,024: x 4.03); valid for the
 # kernel and layout sources whose SHA-256 is recorded with it
 SPMV_TRAFFIC = {

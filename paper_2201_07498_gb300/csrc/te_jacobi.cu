@@ -56,10 +56,7 @@ constexpr int JAC_HALF = MAX_M / 2;
 // element allows (55 blocks); four below 37, where eight are no faster (m = 32:
 // 435 us on either; m = 40: 562 on four, 534 on eight) and take the serving
 // engine's SMs.  Eight hold the 62 blocks per CTA of m = 64.
-#ifndef JAC_CLUSTER4_MIN_M
-#define JAC_CLUSTER4_MIN_M 23
-#define JAC_CLUSTER8_MIN_M 37
-#endif
+constexpr int JAC_CLUSTER4_MIN_M = 23, JAC_CLUSTER8_MIN_M = 37;
 
 TE_DEV uint32_t cluster_ctarank() {
   uint32_t r;

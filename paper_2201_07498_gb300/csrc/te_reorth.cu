@@ -1624,8 +1624,9 @@ cudaError_t launch_batch_pass(int mode, const BatchTable* T, int restart, const 
 // largest, so both bounds leave the sum over j.  A = sixteen outputs' digit j by
 // sixteen columns, from shared memory in fragment order; B = sixteen columns' digit
 // i by eight rows, from registers.  The products with i + j = s share one
-// accumulator: with s from 6 to 14 what is left out lies below 2^-59 of the
-// product of the two bounds; at most 8 pairs x 64 columns x 2^15 = 2^24 units,
+// accumulator: with s from 6 to 14 what is left out lies below 2^-58.4 of the
+// product of the two bounds (64 columns; a bound is a power of two, at most four
+// times the largest element); at most 8 pairs x 64 columns x 2^15 = 2^24 units,
 // exact in binary32.  A row's sums go through 128-bit integers to binary64 with
 // one rounding, by integer instructions.  A row with an infinity or NaN, and
 // coefficients or norms that are not finite or far from 1 (2^-823 ... 2^877), take
