@@ -324,8 +324,7 @@ __global__ void __launch_bounds__(NOALLOC_THREADS, 3) noalloc_chunk_kernel(
   int4 mk[G];
 #pragma unroll
   for (int g = 0; g < G; ++g) mk[g] = reinterpret_cast<const int4*>(sm.mark + tid * Sm::MRUN)[g];
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
+  auto walk = [&](int g, NaSeg<P>& seg, NaAcc<P>& before) {  // four entries
     typename Sm::Pair16 w[4 / Sm::PPV];
 #pragma unroll
     for (int u = 0; u < 4 / Sm::PPV; ++u)
@@ -336,20 +335,44 @@ __global__ void __launch_bounds__(NOALLOC_THREADS, 3) noalloc_chunk_kernel(
       if (4 * g + u < cnt) {
         const int32_t row = u == 0 ? mk[g].x : u == 1 ? mk[g].y : u == 2 ? mk[g].z : mk[g].w;
         if (row >= 0) {
-          if (mine.row >= 0) y[mine.row] = mine.acc.value();
-          else head = mine.acc;
-          mine.acc = NaAcc<P>();
-          mine.row = row;
+          if (seg.row >= 0) y[seg.row] = seg.acc.value();
+          else before = seg.acc;
+          seg.acc = NaAcc<P>();
+          seg.row = row;
         }
         const typename Sm::Pair p = w[u / Sm::PPV].p[u % Sm::PPV];
-        mine.acc.add_prod(p.v, p.x);
+        seg.acc.add_prod(p.v, p.x);
       }
+    }
+  };
+  if constexpr (P == PREC_FDF) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) walk(g, mine, head);
+  } else {
+    // two chains of four, joined: a chain of eight rounds more often than the sum
+    // of a row by a tree (rows of 20 entries: error 1.69e-16 against 1.58e-16)
+    static_assert(P == PREC_FDF || G == 2, "");
+    NaSeg<P> part;
+    NaAcc<P> between;
+    walk(0, mine, head);
+    walk(1, part, between);
+    NaAcc<P> t = mine.acc;
+    t.merge(part.row < 0 ? part.acc : between);
+    if (part.row < 0) {
+      mine.acc = t;
+    } else {
+      if (mine.row >= 0) y[mine.row] = t.value();
+      else head = t;
+      mine = part;
     }
   }
   // inclusive segmented scan over the warp, then what lies before this thread
   NaSeg<P> inc = mine;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
+    // (short rows: no sum reaches further; the vote is cheaper than a merge:
+    // uniform rows of 24 entries, 36.8 M of them, binary64 403 -> 366 us)
+    if (!__any_sync(0xffffffffu, lane >= d && inc.row < 0)) break;
     NaSeg<P> p;
     p.acc = inc.acc.up(d);
     p.row = __shfl_up_sync(0xffffffffu, inc.row, d);
@@ -445,7 +468,9 @@ __global__ void __launch_bounds__(256) noalloc_fixup_kernel(const int64_t* rp, d
 
 // Above this many chunks the rows are searched beforehand (three launches
 // instead of two): a chunk kernel of a few waves hides its own search, and a
-// launch costs about 2 us.
+// launch costs about 2 us.  us a call without and with the search: binary32
+// values 660 chunks 72 and 74, 1,380 89 and 91, 2,100 103 and 103, 4,500 164 and 155,
+// 18,000 514 and 445; binary64 660 63 and 68, from 2,100 to 18,000 within 3 %.
 constexpr int64_t NA_SEARCH_CHUNKS = 2048;
 
 // one call's launches; the chunk kernel's shared memory (above the 48 KB
