@@ -237,7 +237,7 @@ TE_DEV double acc_to_double(typename PassTr<P>::acc_t a) {
 // R-MAT 2^22, 16 columns on average: the delayed form's update 284 -> 125 us
 // (5.25 TB/s; the binary64 pipe was 83 % busy at 27 % of the DRAM peak), the
 // solve 40.5 -> 34.9 ms; the Lanczos phase of 2^19 rows and 40 steps with both
-// sweeps 9.58 -> 8.46 ms.  Error against 64 bits unchanged (4.3e-14 and 5.0e-14
+// sweeps 9.58 -> 8.41 ms.  Error against 64 bits unchanged (4.3e-14 and 5.0e-14
 // for the former's vectors, 1.2e-15 for the latter's basis).
 // From four columns and two tiles per CTA on: the search and the norm's sum
 // cost a CTA about 1 us per step, what they save comes with every tile.  Solves with
