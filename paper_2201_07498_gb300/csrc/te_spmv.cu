@@ -186,24 +186,33 @@ constexpr int SPMV_WPB = 8;     // warps (slices) per CTA
 // with rows relabelled by degree, the first HOT_BYTES of x (the most
 // connected columns) are the ones L1 keeps
 constexpr int64_t HOT_BYTES = 128 << 10;
-// Two forms of the kernel: WIDE has eight entries per lane in flight and free
-// registers, MANY four entries and registers held to six or eight CTAs per SM.
-// The order of a row's sum is the same (entries alternate between two chains).
-// With the gathers split into hot and cold columns (rows by degree) MANY hides
-// their latency better once its warps are all at work: R-MAT 2^22, 128 M entries,
-// us per SpMV, WIDE / MANY: DDD 431 / 375, FDF 291 / 286, 8DF 313 / 282.  In the
-// caller's order, and with too few slices for the warps to fill, a slice's own
-// chain of chunks sets the end: WIDE / MANY, caller's order, R-MAT, 32 entries per
-// row, 50,000 rows FDF 18.8 / 25.0, DDD 21.0 / 24.9, 300,000 rows DDD 44.8 / 55.8,
-// BDF 42.2 / 46.3, 1.5 M rows within 4 %; by degree, R-MAT and uniform rows, slices per
-// SM: DDD 41-62 0.91-1.08 times WIDE's speed, 80-113 1.09-1.14, 156-308 1.04-1.16; binary32
-// arithmetic 40-62 0.93-1.08, 80-113 0.92-1.00, 156-164 1.00-1.12, 283-308 1.01-1.16.
+// Two forms of the kernel: WIDE has eight entries per lane in flight, MANY four and
+// registers held to six (binary64) or eight CTAs per SM.  The order of a row's
+// sum is the same (entries alternate between two chains).  With few slices a
+// slice's own chain of chunks sets the end, and WIDE's is half as long; with many,
+// MANY's warps hide more of the latency, above all where the gathers are split into
+// hot and cold columns (rows by degree) or the matrix streams (x reads local).
+// us per SpMV, WIDE / MANY (R-MAT: 32 entries per row, banded: 16):
+//   by degree    R-MAT 2^22 DDD 431 / 375, FDF 291 / 286, 8DF 313 / 282; 50,000 rows FDF
+//                29.1 / 33.5, DDD 30.9 / 37.0; slices per SM where they meet: DDD 62
+//                (0.91-0.96 of WIDE's speed) to 80 (1.11-1.14), binary32
+//                arithmetic 113 (0.93-1.00) to 156 (1.00-1.12)
+//   caller's     50,000 rows R-MAT FDF 18.8 / 25.0, DDD 21.0 / 24.9; 300,000 DDD 44.8 /
+//                55.8, BDF 42.2 / 46.3; 1.5 M (308 slices per SM) DDD 171 / 174, BDF
+//                157 / 160, 3 M within 1.5 %; banded 1 M rows (206) DDD 50.6 / 45.1, BDF
+//                30.9 / 30.1; 4 M DDD 179 / 157, BDF 106 / 99, 8DF 106 / 100, FDF 108 / 108
+// WIDE's binary32 forms are held to six CTAs: free, they take 46 and 48 registers and
+// stream at five (8DF banded, 12 M rows: 349 us against 304; MANY 280).
 constexpr int SPMV_WIDE = 8, SPMV_MANY = 4;
 constexpr int spmv_ctas_per_sm(int prec, int unroll) {
-  return unroll == SPMV_WIDE ? 1 : prec == PREC_DDD ? 6 : 8;
+  if (unroll == SPMV_WIDE) return prec == PREC_DDD ? 1 : 6;
+  return prec == PREC_DDD ? 6 : 8;
 }
-// MANY from this many slices per SM on, rows by degree
-constexpr int spmv_many_slices(int prec) { return prec == PREC_DDD ? 72 : 128; }
+// MANY from this many slices per SM on
+constexpr int spmv_many_slices(int prec, bool by_degree) {
+  if (by_degree) return prec == PREC_DDD ? 72 : 128;
+  return prec == PREC_DDD ? 256 : 512;
+}
 
 // stored matrix value type per te_dtype, and its streaming load + exact
 // conversion to the arithmetic's input type
@@ -401,7 +410,7 @@ static cudaError_t launch_spmv_t(const SpmvArgs& a, const DevSell& S, cudaStream
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const bool many = a.hot > 0 && S.nslices / sms >= spmv_many_slices(P);
+    const bool many = S.nslices / sms >= spmv_many_slices(P, a.hot > 0);
     auto* k = many ? spmv_kernel<P, VK, F64OUT, SPMV_MANY> : spmv_kernel<P, VK, F64OUT, SPMV_WIDE>;
     k<<<(S.nslices + SPMV_WPB - 1) / SPMV_WPB, 32 * SPMV_WPB, 0, s>>>(a);
   }

@@ -1,7 +1,7 @@
 """The SpMV's two forms (eight entries per lane in flight, or four and more
 CTAs): rows by degree take the second from 72 (binary64) or 128 (binary32)
-slices of 32 rows per SM on, the caller's order always the first.  Row counts on
-either side, rows of 0 ... 20 entries: two steps of the Lanczos phase agree
+slices of 32 rows per SM on, the caller's order from 256 or 512.  Row counts on
+either side of each, rows of 0 ... 20 entries: two steps of the Lanczos phase agree
 between the orders within the summation bound of a row (20 products) and of the
 dots' own rounding."""
 import numpy as np
@@ -20,7 +20,8 @@ def te():
     return te
 
 
-@pytest.mark.parametrize("prec,per_sm,u", [("ddd", 72, 2.0 ** -53), ("fdf", 128, 2.0 ** -24)])
+@pytest.mark.parametrize("prec,per_sm,u", [("ddd", 72, 2.0 ** -53), ("fdf", 128, 2.0 ** -24),
+                                           ("ddd", 256, 2.0 ** -53), ("fdf", 512, 2.0 ** -24)])
 @pytest.mark.parametrize("side", [-3, 3])
 def test_forms_agree(te, prec, per_sm, u, side):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
