@@ -352,7 +352,7 @@ TE_DEV void low_coefs(const PassArgs& a, LowCoef* lc, int* info, int lane) {
 //     when the vector's bound grows.
 // Infinities and NaN have no digits: the dots of a vector or column that holds one
 // are NaN.  Bound by instruction issue and latency, not by the tensor pipe
-// (2^21 rows x 14 columns: ALU 49 % busy, tensor 14 %, DRAM 30 %); two warps per
+// (2^21 rows x 21 columns: ALU 51 % busy, tensor 15 %, DRAM 29 %); two warps per
 // scheduler have registers for it, twice the warps at 96 registers were slower
 // (the pass over 2^22 rows 227 -> 256 us).  With eight-bit integer mma.sync the
 // digits need fewer instructions, but m16n8k32 takes 65 cycles per scheduler on
